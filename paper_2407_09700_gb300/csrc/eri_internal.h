@@ -85,6 +85,10 @@ struct ClassDesc {
   const uint32_t* xytab;       // [products] ix | iy << 8
   const uint32_t* passinfo;    // [xy_npass][2] first product, products in the pass
   int ncomb;                   // distinct products of the class
+  int tiles;                   // fixed-point assembly (eri_fixed.cu): tiles per lane and pass; tables then: outidx [tile][2] words
+                               // x0 | y0 << 8 | x1 << 16 | y1 << 24, z0 | z1 << 16; dst [tile][4] E0
+                               // positions of (x0 y0, z0), (x1 y1, z0), (x0 y0, z1), (x1 y1, z1),
+                               // 0xffffffff for padding; tiles in the order [pass][tile][lane]
   int stage;                   // 1: stage each team's bra / ket PrimPair records into shared memory
                                // by bulk copy (tuning override; kernels compiled for the class only)
   // offsets of the tables in the class's block of the device table (host bookkeeping)
@@ -232,6 +236,12 @@ int erik_upload_cart_tables_small(void);
 int erik_small_available(int la, int lb, int lc, int ld, int fp32);
 int erik_small_blocks_per_sm(int la, int lb, int lc, int ld, int fp32, int* out);
 int erik_launch_small(int la, int lb, int lc, int ld, int fp32, const struct KernelArgs* a, int grid, void* stream);
+// class kernels with the fixed-point assembly (eri_fixed.cu): instantiated lanes per quartet and
+// tiles per lane and pass
+int erik_upload_cart_tables_fixed(void);
+int erik_fixed_variant(int i, int* ts, int* tiles);
+int erik_fixed_blocks_per_sm(int ts, int tiles, int smem_bytes, int* out);
+int erik_launch_fixed(int ts, int tiles, const struct KernelArgs* a, int grid, int smem_bytes, void* stream);
 // energy-gradient class kernels (eri_grad.cu)
 int erik_upload_cart_tables_grad(void);
 int erik_grad_blocks_per_sm(int ts, int smem_bytes, int* out);

@@ -16,12 +16,14 @@
 #include <cstdlib>
 #include <cstring>
 #include <limits>
+#include <map>
 #include <mutex>
 #include <new>
 #include <string>
 #include <vector>
 
 #include "../../include/eri.h"
+#include "eri_fixed.cuh"
 #include "eri_internal.h"
 #include "rys_table.h"
 
@@ -89,6 +91,10 @@ struct DeviceState {
   uint32_t* outidx = nullptr;        // all 225 class index tables
   ClassDesc classes[ERI_NPAIRTYPE][ERI_NPAIRTYPE];
   int ts[ERI_NPAIRTYPE][ERI_NPAIRTYPE];
+  // the same classes for FP64 J/K launches with the fixed-point assembly; fts = 0: none (the
+  // class runs one lane per quartet, or the FP64 class kernel by a tuning override)
+  ClassDesc fclasses[ERI_NPAIRTYPE][ERI_NPAIRTYPE];
+  int fts[ERI_NPAIRTYPE][ERI_NPAIRTYPE];
   uint32_t* grad_outidx = nullptr;   // all gradient class index tables
   GradDesc gclasses[ERI_NPAIRTYPE][ERI_NPAIRTYPE];
   int gts[ERI_NPAIRTYPE][ERI_NPAIRTYPE];
@@ -153,7 +159,7 @@ int team_stride(int doubles, int ts, bool f32) {
 // "la lb lc ld ts xy [stage]" entries separated by ';' in ERI_CLASS_CONFIG (xy -1 = automatic;
 // stage 1 = bulk-copy staging, where a kernel compiled for the class has it), read once per
 // process.  For tuning the choices on new hardware.
-struct ClassTune { int ts = -1, xy = -1, stage = 0; };
+struct ClassTune { int ts = -1, xy = -1, stage = 0; bool overridden = false; };
 ClassTune class_tune(int la, int lb, int lc, int ld) {
   static std::vector<std::vector<int>> table;
   static bool read = false;
@@ -191,6 +197,7 @@ ClassTune class_tune(int la, int lb, int lc, int ld) {
       if (v[4] == 1 || v[4] == 2 || v[4] == 4 || v[4] == 8 || v[4] == 32 || v[4] == 128) t.ts = v[4];
       t.xy = v[5];
       t.stage = v[6] == 1 ? 1 : 0;
+      t.overridden = true;
     }
   return t;
 }
@@ -199,10 +206,10 @@ ClassTune class_tune(int la, int lb, int lc, int ld) {
 // split until every group size occurs a multiple of T times (a leftover group of size
 // s > 1 becomes s-1 and 1; a leftover of single values is padded) and dealt out so that
 // each lane of a T-lane team gets one group of each program entry.  Out: slot_val[o] =
-// value index or -1 (padding) for slot o = (k / 32) * 32 T + (k % 32) * T + lane of the
-// lane's k-th slot; gm[pass] bit k % 32 set where slot k starts a group (every pass starts
-// one); *slots_per_lane.
-void lane_programs(const std::vector<int>& key, int T, std::vector<int>* slot_val, std::vector<uint32_t>* gm,
+// value index or -1 (padding) for slot o = (k / G) * G T + (k % G) * T + lane of the
+// lane's k-th slot (G slots per pass); gm[pass] bit k % G set where slot k starts a group
+// (every pass starts one); *slots_per_lane.
+void lane_programs(const std::vector<int>& key, int T, int G, std::vector<int>* slot_val, std::vector<uint32_t>* gm,
                    int* slots_per_lane) {
   std::vector<std::pair<int, int>> kv;
   for (int v = 0; v < (int)key.size(); ++v) kv.push_back({key[v], v});
@@ -242,20 +249,20 @@ void lane_programs(const std::vector<int>& key, int T, std::vector<int>* slot_va
   }
   int Ls = 0;
   for (int sz : prog) Ls += sz;
-  const int npass = (Ls + 31) / 32;
-  slot_val->assign((size_t)npass * 32 * T, -1);
+  const int npass = (Ls + G - 1) / G;
+  slot_val->assign((size_t)npass * G * T, -1);
   slot_val->resize((size_t)Ls * T);
   gm->assign(npass, 0u);
   int k = 0;
   for (int sz : prog) {
-    (*gm)[k / 32] |= 1u << (k % 32);
+    (*gm)[k / G] |= 1u << (k % G);
     k += sz;
   }
   for (int p = 0; p < npass; ++p) (*gm)[p] |= 1u;
   for (int ln = 0; ln < T; ++ln) {
     int kk = 0;
     for (const auto& g : lane[ln])
-      for (size_t m = 0; m < g.size(); ++m, ++kk) (*slot_val)[(kk / 32) * 32 * T + (kk % 32) * T + ln] = g[m];
+      for (size_t m = 0; m < g.size(); ++m, ++kk) (*slot_val)[(kk / G) * G * T + (kk % G) * T + ln] = g[m];
   }
   *slots_per_lane = Ls;
 }
@@ -333,7 +340,7 @@ void make_class(int la, int lb, int lc, int ld, ClassDesc* c, int* ts, std::vect
     std::vector<int> sv;
     std::vector<uint32_t> gm;
     int Ls = 0;
-    lane_programs(key, T, &sv, &gm, &Ls);
+    lane_programs(key, T, 32, &sv, &gm, &Ls);
     c->nslot = Ls * T;
     c->npass = (int)gm.size();
     std::vector<uint32_t> outi(c->nslot, 1u << 31), dst(c->nslot, 0);
@@ -442,6 +449,101 @@ void make_class(int la, int lb, int lc, int ld, ClassDesc* c, int* ts, std::vect
   if (multi) c->scratch_per_team += ((long long)std::max(c->nslot, c->nout) + 1) / 2 * 2;
 }
 
+// Shared-memory doubles per team of the fixed-point kernels: three blocks per SM.
+int fixed_budget(int ts) { return 8800 * ts / 128; }
+
+// Tiles of the fixed-point assembly (eri_fixed.cu): value v is the product of the I_x I_y entry
+// pair xy[v] and the I_z entry z[v] (each pair of entries at most once).  Pairs with the same
+// list of I_z entries form a rectangle of values, cut into tiles of two pairs by two I_z; a rectangle's odd
+// row or column repeats an entry and its surplus values are padding.
+struct Tile { uint32_t w[2], dst[4]; };
+std::vector<Tile> make_tiles(const std::vector<uint32_t>& xy, const std::vector<uint32_t>& z) {
+  std::map<uint32_t, std::vector<std::pair<uint32_t, uint32_t>>> rows;      // pair -> (z, value)
+  for (size_t v = 0; v < xy.size(); ++v) rows[xy[v]].push_back({z[v], (uint32_t)v});
+  std::map<std::vector<uint32_t>, std::vector<uint32_t>> rect;              // z list -> pairs
+  for (auto& r : rows) {
+    std::sort(r.second.begin(), r.second.end());
+    std::vector<uint32_t> zs;
+    for (auto& q : r.second) zs.push_back(q.first);
+    rect[zs].push_back(r.first);
+  }
+  std::vector<Tile> out;
+  for (auto& r : rect) {
+    const auto& zs = r.first;
+    const auto& ps = r.second;
+    for (size_t i = 0; i < ps.size(); i += 2)
+      for (size_t k = 0; k < zs.size(); k += 2) {
+        const bool two_p = i + 1 < ps.size(), two_z = k + 1 < zs.size();
+        const uint32_t p0 = ps[i], p1 = two_p ? ps[i + 1] : p0, z0 = zs[k], z1 = two_z ? zs[k + 1] : z0;
+        Tile t;
+        t.w[0] = p0 | (p1 << 16);
+        t.w[1] = z0 | (z1 << 16);
+        t.dst[0] = rows[p0][k].second;
+        t.dst[1] = two_p ? rows[p1][k].second : 0xffffffffu;
+        t.dst[2] = two_z ? rows[p0][k + 1].second : 0xffffffffu;
+        t.dst[3] = two_p && two_z ? rows[p1][k + 1].second : 0xffffffffu;
+        out.push_back(t);
+      }
+  }
+  return out;
+}
+
+// The class for FP64 launches with the fixed-point assembly (eri_fixed.cu): team size, tiles,
+// batch and shared-memory layout.  *ts = 0 when the class has no such launch.
+void make_fixed_class(int la, int lb, int lc, int ld, ClassDesc* c, int* ts, std::vector<uint32_t>* idx) {
+  int ts64;
+  make_class(la, lb, lc, ld, c, &ts64, idx);
+  idx->clear();
+  *ts = 0;
+  if (ts64 == 1 || c->Le + c->Lf > FX_LMAX || class_tune(la, lb, lc, ld).overridden) return;
+  const CartTab& ct = cart();
+  const int L1 = c->Lf + 1;
+  std::vector<uint32_t> xy(c->nout), z(c->nout);
+  for (int v = 0; v < c->nout; ++v) {
+    const int e = c->e_base + v / c->nf, f = c->f_base + v % c->nf;
+    xy[v] = (uint32_t)(ct.lx[e] * L1 + ct.lx[f]) | ((uint32_t)(ct.ly[e] * L1 + ct.ly[f]) << 8);
+    z[v] = (uint32_t)(ct.lz[e] * L1 + ct.lz[f]);
+  }
+  std::vector<Tile> tiles = make_tiles(xy, z);
+  // the instantiation that runs the fewest tiles, padding included; of equal ones the larger
+  // team (longer batches)
+  long long best = -1;
+  for (int i = 0, t, nt; erik_fixed_variant(i, &t, &nt); ++i) {
+    const long long np = ((long long)tiles.size() + t * nt - 1) / (t * nt), run = np * t * nt;
+    if (best < 0 || run < best || (run == best && t > *ts)) {
+      best = run;
+      *ts = t;
+      c->tiles = nt;
+      c->npass = (int)np;
+    }
+  }
+  const int T = *ts;
+  c->xy = 0;
+  c->stage = 0;
+  Tile none;
+  none.w[0] = none.w[1] = 0;
+  for (uint32_t& d : none.dst) d = 0xffffffffu;
+  tiles.resize((size_t)best, none);
+  c->nslot = (int)best * 4;
+  c->xysum = (int)best * 2;
+  for (const Tile& t : tiles) idx->insert(idx->end(), t.w, t.w + 2);
+  while (idx->size() % 4) idx->push_back(0);
+  c->dst_off = (int)idx->size();
+  for (const Tile& t : tiles) idx->insert(idx->end(), t.dst, t.dst + 4);
+  c->gmask_off = 0;
+  c->nIs = c->nI | 1;
+  // per primitive quartet 22 scalars and three tables per root, per team K of the 3 nI entries
+  // and of the steps
+  const int per_prim = 4 + 18 + 3 * c->nroots * c->nIs, fixed = (3 * c->nI + FX_TERMS + 1) / 2;
+  c->bp = std::max(1, std::min(FX_TERMS / c->nroots, (fixed_budget(T) - fixed) / per_prim));
+  c->team_doubles = team_stride(c->bp * per_prim + fixed, T, false);
+  c->team_doubles_xy = c->team_doubles_f32 = c->bp_xy = 0;
+  c->split3 = choose_split3(T, c->bp, c->nroots, c->nI, 0);
+  c->scratch_per_team = ((long long)c->nout + 1) / 2 * 2 + 2LL * c->hrr_doubles;
+  c->part_off = c->scratch_per_team;
+  c->scratch_per_team += ((long long)c->nslot + 1) / 2 * 2;
+}
+
 // Fill the static part of a gradient class descriptor (Sec. 4): the four contracted sets,
 // their 2D-table offsets tagged with the set, team sizes and the scratch layout.
 void make_grad_class(int la, int lb, int lc, int ld, GradDesc* g, int* ts, std::vector<uint32_t>* idx) {
@@ -487,7 +589,7 @@ void make_grad_class(int la, int lb, int lc, int ld, GradDesc* g, int* ts, std::
   std::vector<int> sv;
   std::vector<uint32_t> gm;
   int Ls = 0;
-  lane_programs(key, *ts, &sv, &gm, &Ls);
+  lane_programs(key, *ts, 32, &sv, &gm, &Ls);
   g->nslot = Ls * *ts;
   g->npass = (int)gm.size();
   std::vector<uint32_t> dst(g->nslot, 0);
@@ -543,6 +645,7 @@ eri_status device_init(int dev, DeviceState** out) {
     CUDA_TRY(erik_upload_cart_tables_small());
     CUDA_TRY(erik_upload_cart_tables_grad());
     CUDA_TRY(erik_upload_cart_tables_spec());
+    CUDA_TRY(erik_upload_cart_tables_fixed());
     CUDA_TRY(erik_class_spec_prepare());
     size_t ncoef = (size_t)RYS_NCOEF, nas = (size_t)RYS_ASYM_OFFSET[RYS_NMAX] + RYS_NMAX;
     CUDA_TRY(cudaMalloc(&s.rys_coef, sizeof(double) * ncoef));
@@ -552,7 +655,7 @@ eri_status device_init(int dev, DeviceState** out) {
     CUDA_TRY(cudaMemcpy(s.rys_au, RYS_ASYM_U, sizeof(double) * nas, cudaMemcpyHostToDevice));
     CUDA_TRY(cudaMemcpy(s.rys_aw, RYS_ASYM_W, sizeof(double) * nas, cudaMemcpyHostToDevice));
     std::vector<uint32_t> all, one;
-    size_t offs[ERI_NPAIRTYPE][ERI_NPAIRTYPE];
+    size_t offs[ERI_NPAIRTYPE][ERI_NPAIRTYPE], foffs[ERI_NPAIRTYPE][ERI_NPAIRTYPE];
     for (int X = 0; X < ERI_NPAIRTYPE; ++X)
       for (int Y = 0; Y < ERI_NPAIRTYPE; ++Y) {
         int la, lb, lc, ld;
@@ -560,6 +663,10 @@ eri_status device_init(int dev, DeviceState** out) {
         ptype_ls(Y, &lc, &ld);
         make_class(la, lb, lc, ld, &s.classes[X][Y], &s.ts[X][Y], &one);
         offs[X][Y] = all.size();
+        all.insert(all.end(), one.begin(), one.end());
+        make_fixed_class(la, lb, lc, ld, &s.fclasses[X][Y], &s.fts[X][Y], &one);
+        while (all.size() % 4) all.push_back(0);       // read as 16-byte words
+        foffs[X][Y] = all.size();
         all.insert(all.end(), one.begin(), one.end());
       }
     CUDA_TRY(cudaMalloc(&s.outidx, sizeof(uint32_t) * all.size()));
@@ -577,6 +684,10 @@ eri_status device_init(int dev, DeviceState** out) {
           cd.xytab = base + cd.xytab_off;
           cd.passinfo = base + cd.pass_off;
         }
+        ClassDesc& fd = s.fclasses[X][Y];
+        fd.outidx = s.outidx + foffs[X][Y];
+        fd.dst = fd.outidx + fd.dst_off;
+        fd.gmask = fd.outidx + fd.gmask_off;
       }
     all.clear();
     for (int X = 0; X < ERI_NPAIRTYPE; ++X)
@@ -736,7 +847,7 @@ struct eri_plan {
   bool profiling = false;
   std::vector<cudaEvent_t> events;            // 2 per launch
   std::vector<int> last_launch_xy;            // X*15+Y per launch
-  std::vector<int> last_launch_ts, last_launch_grid, last_launch_fp32, last_launch_small;
+  std::vector<int> last_launch_ts, last_launch_grid, last_launch_fp32, last_launch_small, last_launch_fixed;
   std::vector<int> last_launch_qsplit, last_launch_listed;
 };
 
@@ -769,11 +880,12 @@ eri_status ensure_buf(T** ptr, size_t* cap, size_t n) {
   return ERI_OK;
 }
 
-// Grid and dynamic shared memory for one class launch.
-eri_status launch_shape(eri_plan* p, int X, int Y, int fp32, long long nteams_needed, int* grid, int* smem,
+// Grid and dynamic shared memory for one class launch: of the FP64 or FP32 class kernel, or
+// (fixed) of the FP64 launch with the fixed-point assembly.
+eri_status launch_shape(eri_plan* p, int X, int Y, int fp32, int fixed, long long nteams_needed, int* grid, int* smem,
                         int* ts_out) {
-  const ClassDesc& c = p->dev->classes[X][Y];
-  const int ts = p->dev->ts[X][Y];
+  const ClassDesc& c = fixed ? p->dev->fclasses[X][Y] : p->dev->classes[X][Y];
+  const int ts = fixed ? p->dev->fts[X][Y] : p->dev->ts[X][Y];
   const int teams_per_block = 128 / ts;
   *smem = (int)(sizeof(double) * (size_t)(fp32 ? c.team_doubles_f32 : (c.xy ? c.team_doubles_xy : c.team_doubles)) *
                 teams_per_block);
@@ -781,7 +893,10 @@ eri_status launch_shape(eri_plan* p, int X, int Y, int fp32, long long nteams_ne
   if (c.stage && !fp32) *smem = ((*smem + 15) & ~15) + teams_per_block * (20 * (int)sizeof(PrimPair) + 8);
   if (*smem > 200 * 1024) return fail(ERI_ERR_ARG, "class (%d%d|%d%d) needs %d bytes of shared memory", c.la, c.lb, c.lc, c.ld, *smem);
   int bps = 0;
-  CUDA_TRY(erik_blocks_per_sm(ts, fp32, (c.xy && !fp32) ? 1 : 0, *smem, &bps));
+  if (fixed)
+    CUDA_TRY(erik_fixed_blocks_per_sm(ts, c.tiles, *smem, &bps));
+  else
+    CUDA_TRY(erik_blocks_per_sm(ts, fp32, (c.xy && !fp32) ? 1 : 0, *smem, &bps));
   if (bps < 1) bps = 1;
   long long full = (long long)p->dev->sms * bps;
   long long need = (nteams_needed + teams_per_block - 1) / teams_per_block;
@@ -818,7 +933,7 @@ eri_status run_explicit(eri_plan* p, int X, int Y, int mode, const std::vector<i
   if ((s = ensure_buf(&p->d_out, &p->out_cap, std::max<size_t>(out_doubles, 1))) != ERI_OK) return s;
   if (mode == KMODE_BLOCK && (s = ensure_buf(&p->d_off, &p->off_cap, offs.size())) != ERI_OK) return s;
   int grid, smem, ts;
-  if ((s = launch_shape(p, X, Y, 0, nt, &grid, &smem, &ts)) != ERI_OK) return s;
+  if ((s = launch_shape(p, X, Y, 0, 0, nt, &grid, &smem, &ts)) != ERI_OK) return s;
   const ClassDesc& c = p->dev->classes[X][Y];
   size_t need = (size_t)grid * (size_t)(128 / ts) * (size_t)c.scratch_per_team;
   if ((s = ensure_scratch(p, need)) != ERI_OK) return s;
@@ -872,7 +987,12 @@ struct Launch {
   int small;             // 1: compile-time specialised kernel (eri_small.cu)
   int split;             // 1: the class runs an FP64 and an FP32 launch (mixed mode)
   int qsplit;            // tasks per quartet (ranges of its primitive quartets), 1 = none
+  int fixed;             // 1: FP64 launch with the fixed-point assembly (eri_fixed.cu)
 };
+
+const ClassDesc& launch_class(const eri_plan* p, const Launch& l) {
+  return l.fixed ? p->dev->fclasses[l.X][l.Y] : p->dev->classes[l.X][l.Y];
+}
 
 // Classes with at most this many candidate quartets screen in the kernel instead of being
 // compacted first (three launches saved per class on small molecules).
@@ -890,6 +1010,40 @@ int choose_qsplit(long long nt, long long teams, int maxq, int minq) {
   if (nt <= 0 || maxq <= minq || nt * 2 > teams) return 1;
   const long long q = (teams + nt - 1) / nt;
   return (int)std::max(1LL, std::min<long long>({q, (long long)(maxq / std::max(1, minq)), 64LL}));
+}
+
+// Kernel, split, grid and shared memory of a J/K launch over l->nt candidate quartets of at most
+// maxq primitive quartets: the specialised one-lane kernel where the class runs with one lane
+// per quartet (FP32: whenever one exists), else for FP64 the fixed-point assembly where the
+// class has one, else the FP64 / FP32 class kernel.
+eri_status shape_launch(eri_plan* p, int maxq, Launch* l) {
+  const ClassDesc& cd = p->dev->classes[l->X][l->Y];
+  if ((l->fp32 || p->dev->ts[l->X][l->Y] == 1) && erik_small_available(cd.la, cd.lb, cd.lc, cd.ld, l->fp32)) {
+    int bps = 0;
+    CUDA_TRY(erik_small_blocks_per_sm(cd.la, cd.lb, cd.lc, cd.ld, l->fp32, &bps));
+    const long long full = (long long)p->dev->sms * std::max(bps, 1);
+    l->ts = 1;
+    l->qsplit = choose_qsplit(l->nt, full * 128, maxq, 2);
+    l->grid = (int)std::max(1LL, std::min(full, (l->nt * l->qsplit + 127) / 128));
+    l->smem = 0;
+    l->small = 1;
+    return ERI_OK;
+  }
+  l->fixed = !l->fp32 && p->dev->fts[l->X][l->Y] > 0;
+  const ClassDesc& c = launch_class(p, *l);
+  // a full grid first: the teams it holds decide the split, the split the grid
+  eri_status s = launch_shape(p, l->X, l->Y, l->fp32, l->fixed, 1LL << 40, &l->grid, &l->smem, &l->ts);
+  if (s != ERI_OK) return s;
+  l->qsplit = choose_qsplit(l->nt, (long long)l->grid * (128 / l->ts), maxq, l->fp32 || !c.xy ? c.bp : c.bp_xy);
+  return launch_shape(p, l->X, l->Y, l->fp32, l->fixed, l->nt * l->qsplit, &l->grid, &l->smem, &l->ts);
+}
+
+// Run the launch's kernel (a.c is set to its class).
+int run_launch(const eri_plan* p, const Launch& l, KernelArgs& a, cudaStream_t st) {
+  a.c = launch_class(p, l);
+  if (l.small) return erik_launch_small(a.c.la, a.c.lb, a.c.lc, a.c.ld, l.fp32, &a, l.grid, st);
+  if (l.fixed) return erik_launch_fixed(l.ts, a.c.tiles, &a, l.grid, l.smem, st);
+  return erik_launch_class(l.ts, l.fp32, &a, l.grid, l.smem, st);
 }
 
 eri_status check_jk_args(eri_plan* p, const double* D, int nD, double* J, double* K, int flags) {
@@ -926,32 +1080,11 @@ eri_status plan_launches(eri_plan* p, size_t max_scratch, std::vector<Launch>* o
       const long long nt = (X == Y) ? nx * (nx + 1) / 2 : nx * ny;
       const int np = (nprec == 2 && fp32_pays(p, X, Y, nt)) ? 2 : 1;
       for (int fp32 = 0; fp32 < np; ++fp32) {
-        Launch l{X, Y, fp32, 0, 0, 0, nt, 0, np == 2 ? 1 : 0, 1};
-        const ClassDesc& cd = p->dev->classes[X][Y];
-        // a full grid first: the teams it holds decide the split, the split the grid
-        eri_status s = launch_shape(p, X, Y, fp32, 1LL << 40, &l.grid, &l.smem, &l.ts);
+        Launch l{X, Y, fp32, 0, 0, 0, nt, 0, np == 2 ? 1 : 0, 1, 0};
+        eri_status s = shape_launch(p, p->type_maxprim[X] * p->type_maxprim[Y], &l);
         if (s != ERI_OK) return s;
-        const int maxq = p->type_maxprim[X] * p->type_maxprim[Y];
-        l.qsplit = choose_qsplit(nt, (long long)l.grid * (128 / l.ts), maxq,
-                                 fp32 ? cd.bp : (cd.xy ? cd.bp_xy : cd.bp));
-        s = launch_shape(p, X, Y, fp32, nt * l.qsplit, &l.grid, &l.smem, &l.ts);
-        if (s != ERI_OK) return s;
-        // specialised one-lane kernel: FP64 when the class runs with one lane per quartet,
-        // FP32 whenever one exists (its accumulators fit a lane in FP32)
-        if ((fp32 || l.ts == 1) && erik_small_available(cd.la, cd.lb, cd.lc, cd.ld, fp32)) {
-          l.ts = 1;
-          int bps = 0;
-          CUDA_TRY(erik_small_blocks_per_sm(cd.la, cd.lb, cd.lc, cd.ld, fp32, &bps));
-          if (bps < 1) bps = 1;
-          const long long full = (long long)p->dev->sms * bps;
-          l.qsplit = choose_qsplit(nt, full * 128, maxq, 2);
-          const long long need = (nt * l.qsplit + 127) / 128;
-          l.grid = (int)std::max(1LL, std::min(full, need));
-          l.smem = 0;
-          l.small = 1;
-        }
         if (max_scratch > 0) {
-          const ClassDesc& c = p->dev->classes[X][Y];
+          const ClassDesc& c = launch_class(p, l);
           const size_t per_block = (size_t)(128 / l.ts) * (size_t)c.scratch_per_team;
           if (per_block > max_scratch)
             return fail(ERI_ERR_ARG,
@@ -1009,6 +1142,7 @@ eri_status run_jk(eri_plan* p, const std::vector<Launch>& launches, const double
   p->last_launch_grid.clear();
   p->last_launch_fp32.clear();
   p->last_launch_small.clear();
+  p->last_launch_fixed.clear();
   p->last_launch_qsplit.clear();
   p->last_launch_listed.clear();
   if (nstreams == 2) {
@@ -1059,10 +1193,7 @@ eri_status run_jk(eri_plan* p, const std::vector<Launch>& launches, const double
       a.tcount = cnt + l.fp32;
     }
     if (prof) CUDA_TRY(cudaEventRecord(p->events[2 * li], sl));
-    if (l.small)
-      CUDA_TRY(erik_launch_small(a.c.la, a.c.lb, a.c.lc, a.c.ld, l.fp32, &a, l.grid, sl));
-    else
-      CUDA_TRY(erik_launch_class(l.ts, l.fp32, &a, l.grid, l.smem, sl));
+    CUDA_TRY(run_launch(p, l, a, sl));
     if (prof) CUDA_TRY(cudaEventRecord(p->events[2 * li + 1], sl));
     if (record) {
       p->last_launch_xy.push_back(l.X * ERI_NPAIRTYPE + l.Y);
@@ -1070,6 +1201,7 @@ eri_status run_jk(eri_plan* p, const std::vector<Launch>& launches, const double
       p->last_launch_grid.push_back(l.grid);
       p->last_launch_fp32.push_back(l.fp32);
       p->last_launch_small.push_back(l.small);
+      p->last_launch_fixed.push_back(l.fixed);
       p->last_launch_qsplit.push_back(l.qsplit);
       p->last_launch_listed.push_back(listed ? 1 : 0);
     }
@@ -1100,7 +1232,7 @@ eri_status size_jk_buffers(eri_plan* p, std::vector<Launch>* launches, size_t* n
   if ((s = plan_launches(p, 0, launches)) != ERI_OK) return s;
   size_t need = 0;
   for (const Launch& l : *launches)
-    need = std::max(need, (size_t)l.grid * (size_t)(128 / l.ts) * (size_t)p->dev->classes[l.X][l.Y].scratch_per_team);
+    need = std::max(need, (size_t)l.grid * (size_t)(128 / l.ts) * (size_t)launch_class(p, l).scratch_per_team);
   need = (need + 31) & ~(size_t)31;
   size_t maxnt = 1;
   for (const Launch& l : *launches)
@@ -1714,8 +1846,9 @@ eri_status eri_launch_records(eri_plan* p, eri_launch_record* out, int cap, int*
     r.model_flops_fp32 = a32 * (double)r.prim_quartets + q32 * (double)r.quartets;
     r.fp32 = f;
     r.specialised = p->last_launch_small[i];
-    r.shared_products = (!f && !r.specialised && c.xy) ? 1 : 0;
-    r.compiled_class = (!f && !r.specialised && erik_class_spec_available(r.team_size, c.la, c.lb, c.lc, c.ld)) ? 1 : 0;
+    const bool cls64 = !f && !r.specialised && !p->last_launch_fixed[i];
+    r.shared_products = (cls64 && c.xy) ? 1 : 0;
+    r.compiled_class = (cls64 && erik_class_spec_available(r.team_size, c.la, c.lb, c.lc, c.ld)) ? 1 : 0;
     r.quartet_split = p->last_launch_qsplit[i];
     r.listed = p->last_launch_listed[i];
   }
@@ -1732,19 +1865,19 @@ eri_status eri_check_class_tables(int* nclasses, int* problems) {
   if (!nclasses || !problems) return fail(ERI_ERR_ARG, "NULL output");
   const CartTab& ct = cart();
   int bad = 0, n = 0;
-  auto check_lp = [&](const uint32_t* outi, const uint32_t* dst, const uint32_t* gm, int T, int nslot, int nval,
+  auto check_lp = [&](const uint32_t* outi, const uint32_t* dst, const uint32_t* gm, int T, int G, int nslot, int nval,
                       auto&& expect) {
     const int Ls = nslot / T;
     if (Ls * T != nslot) ++bad;
     std::vector<int> seen(nval, 0);
-    for (int p = 0; p < (Ls + 31) / 32; ++p)
+    for (int p = 0; p < (Ls + G - 1) / G; ++p)
       if (!(gm[p] & 1u)) ++bad;
     for (int ln = 0; ln < T; ++ln) {
       uint32_t cur = 0xffffffffu;
       for (int k = 0; k < Ls; ++k) {
-        const int o = (k / 32) * T * 32 + (k % 32) * T + ln;
+        const int o = (k / G) * T * G + (k % G) * T + ln;
         const uint32_t q = outi[o];
-        if ((gm[k / 32] >> (k % 32)) & 1u) cur = q & 0xffffu;
+        if ((gm[k / G] >> (k % G)) & 1u) cur = q & 0xffffu;
         if (q >> 31) continue;
         if ((q & 0xffffu) != cur) ++bad;
         if ((int)dst[o] < 0 || (int)dst[o] >= nval) { ++bad; continue; }
@@ -1771,7 +1904,7 @@ eri_status eri_check_class_tables(int* nclasses, int* problems) {
           return (uint32_t)(ct.lx[e] * L1 + ct.lx[f]) | ((uint32_t)(ct.ly[e] * L1 + ct.ly[f]) << 8) |
                  ((uint32_t)(ct.lz[e] * L1 + ct.lz[f]) << 16);
         };
-        check_lp(idx.data(), idx.data() + c.dst_off, idx.data() + c.gmask_off, ts, c.nslot, c.nout,
+        check_lp(idx.data(), idx.data() + c.dst_off, idx.data() + c.gmask_off, ts, 32, c.nslot, c.nout,
                  [&](int v, uint32_t q) { return (q & 0xffffffu) == word(v); });
         const int tpb = 128 / ts;
         if (ts > 1 && (8L * c.team_doubles * tpb > 200 * 1024 || 8L * c.team_doubles_f32 * tpb > 200 * 1024)) ++bad;
@@ -1793,6 +1926,33 @@ eri_status eri_check_class_tables(int* nclasses, int* problems) {
         }
       }
       {
+        ClassDesc c;
+        std::vector<uint32_t> idx;
+        make_fixed_class(la, lb, lc, ld, &c, &ts, &idx);
+        if (ts > 0) {
+          const int L1 = c.Lf + 1, nt = c.nslot / 4;
+          std::vector<int> seen(c.nout, 0);
+          if (nt != c.npass * c.tiles * ts || c.dst_off % 4 || (int)idx.size() != c.dst_off + 4 * nt) ++bad;
+          for (int t = 0; t < nt; ++t)
+            for (int q = 0; q < 4; ++q) {
+              const uint32_t p = (idx[2 * t] >> (16 * (q & 1))) & 0xffffu, zi = (idx[2 * t + 1] >> (16 * (q >> 1))) & 0xffffu;
+              const uint32_t d = idx[c.dst_off + 4 * t + q];
+              if ((int)(p & 0xffu) >= c.nI || (int)(p >> 8) >= c.nI || (int)zi >= c.nI) ++bad;
+              if (d == 0xffffffffu) continue;
+              if ((int)d >= c.nout || seen[d]++) { ++bad; continue; }
+              const int e = c.e_base + (int)d / c.nf, f = c.f_base + (int)d % c.nf;
+              if ((p & 0xffu) != (uint32_t)(ct.lx[e] * L1 + ct.lx[f]) || (p >> 8) != (uint32_t)(ct.ly[e] * L1 + ct.ly[f]) ||
+                  zi != (uint32_t)(ct.lz[e] * L1 + ct.lz[f]))
+                ++bad;
+            }
+          for (int v = 0; v < c.nout; ++v)
+            if (seen[v] != 1) ++bad;
+          if (c.bp * c.nroots > FX_TERMS || 8L * c.team_doubles * (128 / ts) > 200 * 1024) ++bad;
+          const int ntab = c.bp * 3 * c.nroots * c.nIs;
+          if (8L * c.team_doubles < 8L * c.bp * 22 + 8L * ntab + 4L * (3 * c.nI + c.bp * c.nroots)) ++bad;
+        }
+      }
+      {
         GradDesc g;
         std::vector<uint32_t> idx;
         make_grad_class(la, lb, lc, ld, &g, &ts, &idx);
@@ -1807,7 +1967,7 @@ eri_status eri_check_class_tables(int* nclasses, int* problems) {
                  ((q >> 8) & 0xffu) == (uint32_t)(ct.ly[e] * L1 + ct.ly[f]) &&
                  ((q >> 16) & 0xfffu) == (uint32_t)(set * NnI + ct.lz[e] * L1 + ct.lz[f]);
         };
-        check_lp(idx.data(), idx.data() + g.dst_off, idx.data() + g.gmask_off, ts, g.nslot, g.nout, expect);
+        check_lp(idx.data(), idx.data() + g.dst_off, idx.data() + g.gmask_off, ts, 32, g.nslot, g.nout, expect);
         if (ts > 1 && 8L * g.team_doubles * (128 / ts) > 200 * 1024) ++bad;
       }
     }
@@ -2020,31 +2180,15 @@ eri_status eri_jk_batch(eri_batch* b, int njobs, eri_plan* const* plans, const d
       if (tot) cls.push_back({X, Y, tot, mx, any32, maxq});
     }
   size_t cap = 1, tcap = 2, need = 0;
-  struct LL { int X, Y, fp32, grid, smem, ts, small; long long total; int qsplit; };
-  std::vector<LL> launches;
+  std::vector<Launch> launches;
   for (const BL& c : cls) {
     cap = std::max(cap, (size_t)c.total);
     tcap = std::max(tcap, (size_t)(2 * ((c.maxnt + 1023) / 1024 + 1)));
     for (int fp32 = 0; fp32 < (c.any_fp32 ? 2 : 1); ++fp32) {
-      LL l{c.X, c.Y, fp32, 0, 0, 0, 0, c.total, 1};
-      const ClassDesc& cd = p0->dev->classes[c.X][c.Y];
-      // as in eri_jk: a class whose merged quartets cannot fill the grid splits them into
-      // ranges of primitive quartets (a full grid decides the split, the split the grid)
-      if ((s = launch_shape(p0, c.X, c.Y, fp32, 1LL << 40, &l.grid, &l.smem, &l.ts)) != ERI_OK) return s;
-      l.qsplit = choose_qsplit(c.total, (long long)l.grid * (128 / l.ts), c.maxq,
-                               fp32 ? cd.bp : (cd.xy ? cd.bp_xy : cd.bp));
-      if ((s = launch_shape(p0, c.X, c.Y, fp32, c.total * l.qsplit, &l.grid, &l.smem, &l.ts)) != ERI_OK) return s;
-      if ((fp32 || l.ts == 1) && erik_small_available(cd.la, cd.lb, cd.lc, cd.ld, fp32)) {
-        l.ts = 1;
-        int bps = 0;
-        CUDA_TRY(erik_small_blocks_per_sm(cd.la, cd.lb, cd.lc, cd.ld, fp32, &bps));
-        const long long full = (long long)p0->dev->sms * std::max(bps, 1);
-        l.qsplit = choose_qsplit(c.total, full * 128, c.maxq, 2);
-        l.grid = (int)std::max(1LL, std::min(full, (c.total * l.qsplit + 127) / 128));
-        l.smem = 0;
-        l.small = 1;
-      }
-      need = std::max(need, (size_t)l.grid * (size_t)(128 / l.ts) * (size_t)cd.scratch_per_team);
+      // as in eri_jk, over the jobs' merged quartets
+      Launch l{c.X, c.Y, fp32, 0, 0, 0, c.total, 0, 0, 1, 0};
+      if ((s = shape_launch(p0, c.maxq, &l)) != ERI_OK) return s;
+      need = std::max(need, (size_t)l.grid * (size_t)(128 / l.ts) * (size_t)launch_class(p0, l).scratch_per_team);
       launches.push_back(l);
     }
   }
@@ -2106,7 +2250,7 @@ eri_status eri_jk_batch(eri_batch* b, int njobs, eri_plan* const* plans, const d
       CUDA_TRY(erik_launch_compact_batched(&a, blist_l, (unsigned long long)c.total, small_l, tiles_l, cursor,
                                            small_l + 2, (unsigned long long)j, split ? 1 : 0, sl));
     }
-    for (const LL& l : launches) {
+    for (const Launch& l : launches) {
       if (l.X != c.X || l.Y != c.Y) continue;
       KernelArgs a = base_args(p0, c.X, c.Y);
       a.mode = KMODE_JK;
@@ -2121,10 +2265,7 @@ eri_status eri_jk_batch(eri_batch* b, int njobs, eri_plan* const* plans, const d
       a.scratch = b->d_scratch + (size_t)sidx * need;
       a.qsplit = l.qsplit;
       a.stats = b->d_stats + 2 * (256 * l.fp32 + c.X * ERI_NPAIRTYPE + c.Y);
-      if (l.small)
-        CUDA_TRY(erik_launch_small(a.c.la, a.c.lb, a.c.lc, a.c.ld, l.fp32, &a, l.grid, sl));
-      else
-        CUDA_TRY(erik_launch_class(l.ts, l.fp32, &a, l.grid, l.smem, sl));
+      CUDA_TRY(run_launch(p0, l, a, sl));
       ++li;
     }
   }
