@@ -249,16 +249,10 @@ __global__ void __launch_bounds__(TPB, (TS == 1 ? 3 : ((sizeof(R) == 4 && !XY) ?
           const PrimPair* yd = (STAGE && staged) ? stage + npb + q % npk : tc.prims + iyp;
           const double s = xd->zeta + yd->zeta;
           const double rd = rsqrt(s);
-          const double PQ0 = xd->P[0] - yd->P[0], PQ1 = xd->P[1] - yd->P[1], PQ2 = xd->P[2] - yd->P[2];
+          double PQ0, PQ1, PQ2;
+          pair_distance(tc, xd, yd, ixp, iyp, PQ0, PQ1, PQ2);
           const double T = xd->zeta * yd->zeta * (rd * rd) * fma(PQ0, PQ0, fma(PQ1, PQ1, PQ2 * PQ2));
-          int ti;
-          double xx, invT, rsqT;
-          rys_locate(T, a.rys_tcut_d, ti, xx, invT, rsqT);
-          const int od = j * NPD;
-          sd[od + 0] = xx;
-          sd[od + 1] = invT;
-          sd[od + 2] = rsqT;
-          sd[od + 3] = __longlong_as_double((long long)ti);
+          rys_put_team(sd, j * NPD, rys_locate(T, a.rys_tcut_hi));
           const PP* x = (sizeof(R) == 8) ? reinterpret_cast<const PP*>(xd) : prims_r + ixp;
           const PP* y = (sizeof(R) == 8) ? reinterpret_cast<const PP*>(yd) : prims_r + iyp;
           const R zeta = x->zeta, eta = y->zeta;
@@ -289,17 +283,15 @@ __global__ void __launch_bounds__(TPB, (TS == 1 ? 3 : ((sizeof(R) == 4 && !XY) ?
           const int jn = tk / 3, ax = tk - jn * 3;
           const int j = jn / N, n = jn - (jn / N) * N;
           if (j < nbt) {
-            const int od = j * NPD, o = j * NPR;
-            double ud, wd;
-            rys_root(a.rys_coef, a.rys_au, a.rys_aw, N, (int)__double_as_longlong(sd[od + 3]), sd[od + 0],
-                     sd[od + 1], sd[od + 2], n, ud, wd);
-            const R u = (R)ud;
+            const int o = j * NPR;
+            R u, wd;
+            rys_root(a.rys_coef, a.rys_au, a.rys_aw, N, rys_get_team(sd, j * NPD), n, u, wd);
             const R B00 = u * sr[o + 12];
             const R B10 = fma(-u, sr[o + 13], sr[o + 16]);
             const R B01 = fma(-u, sr[o + 14], sr[o + 17]);
             const R Cax = fma(-u, sr[o + 6 + ax], sr[o + 0 + ax]);
             const R Cpx = fma(u, sr[o + 9 + ax], sr[o + 3 + ax]);
-            const R I00 = (ax == 2) ? (R)wd * sr[o + 15] : R(1);
+            const R I00 = (ax == 2) ? wd * sr[o + 15] : R(1);
             rys_2d1<R>(sr, S_2D + ((j * 3 + ax) * N + n) * nIs, Le, Lf, I00, Cax, Cpx, B00, B10, B01);
           }
         }
@@ -307,15 +299,13 @@ __global__ void __launch_bounds__(TPB, (TS == 1 ? 3 : ((sizeof(R) == 4 && !XY) ?
         for (int tk = tl; tk < bp * N; tk += TS) {
           const int j = tk / N, n = tk - (tk / N) * N;
           if (j < nbt) {
-            const int od = j * NPD, o = j * NPR;
-            double ud, wd;
-            rys_root(a.rys_coef, a.rys_au, a.rys_aw, N, (int)__double_as_longlong(sd[od + 3]), sd[od + 0],
-                     sd[od + 1], sd[od + 2], n, ud, wd);
-            const R u = (R)ud, w = (R)wd;
+            const int o = j * NPR;
+            R u, wd;
+            rys_root(a.rys_coef, a.rys_au, a.rys_aw, N, rys_get_team(sd, j * NPD), n, u, wd);
             const R B00 = u * sr[o + 12];
             const R B10 = fma(-u, sr[o + 13], sr[o + 16]);
             const R B01 = fma(-u, sr[o + 14], sr[o + 17]);
-            const R wt = w * sr[o + 15];
+            const R wt = wd * sr[o + 15];
             const R C[3] = {fma(-u, sr[o + 6], sr[o + 0]), fma(-u, sr[o + 7], sr[o + 1]),
                             fma(-u, sr[o + 8], sr[o + 2])};
             const R Cp[3] = {fma(u, sr[o + 9], sr[o + 3]), fma(u, sr[o + 10], sr[o + 4]),

@@ -6,7 +6,7 @@
 #include <stdint.h>
 
 #include "eri_internal.h"
-#include "rys_table.h"
+#include "rys_fixed.h"
 
 #define TPB 128        // threads per block of the class kernels
 #define GSLOTS 32      // accumulator slots per lane
@@ -46,50 +46,110 @@ struct Smem {
 };
 
 // ------------------------------------------------------------------ Rys roots and weights
-// Degree-RYS_DEG polynomial, highest power first, by Horner's rule.
-__device__ __forceinline__ double horner_rys(const double* __restrict__ c, double x) {
-  double a = __ldg(c);
+// The table lookup of one T: interval ti and position x in it (rys_fixed.h), or ti = -1 and
+// 1 / sqrt(T) in the large-T limit.  tcut_hi: high word of the cutoff (an integer, so the high
+// words decide T < tcut; an infinity or a NaN takes the limit).
+struct RysAt {
+  int ti;
+  int32_t x0;
+  uint32_t x1;
+  double rsqT;
+};
+__device__ __forceinline__ RysAt rys_locate(double T, int tcut_hi) {
+  RysAt r;
+  r.ti = -1;
+  r.x0 = 0;
+  r.x1 = 0;
+  r.rsqT = 0.0;
+  if ((__double2hiint(T) & 0x7fffffff) < tcut_hi)
+    rys_fx_locate((uint64_t)__double_as_longlong(T) & 0x7fffffffffffffffULL, r.ti, r.x0, r.x1);
+  else
+    r.rsqT = rsqrt(T);
+  return r;
+}
+
+// v 2^(E - 62) for v > 0 (v = 0 counts as 1)
+__device__ __forceinline__ double rys_value(int64_t v, int E, double) {
+  const double d = __ll2double_rn(v > 0 ? v : 1);
+  return __hiloint2double(__double2hiint(d) + ((E - 62) << 20), __double2loint(d));
+}
+__device__ __forceinline__ float rys_value(int64_t v, int E, float) {
+  const float f = __ll2float_rn(v > 0 ? v : 1);
+  return __int_as_float(__float_as_int(f) + ((E - 62) << 23));
+}
+
+// Root n of N and its weight, in the recurrence type.
+template <typename R>
+__device__ __forceinline__ void rys_root(const int64_t* __restrict__ coef, const double* __restrict__ au,
+                                         const double* __restrict__ aw, int N, const RysAt& at, int n, R& u, R& w) {
+  if (at.ti >= 0) {
+    const longlong2* c = reinterpret_cast<const longlong2*>(coef) + ((size_t)at.ti * N + n) * (RYS_DEG + 1);
+    int64_t row[RYS_DEG + 1];
+    int E;
 #pragma unroll
-  for (int k = 1; k <= RYS_DEG; ++k) a = fma(a, x, __ldg(c + k));
-  return a;
-}
-
-// floor(T) for 0 <= T < 2^30 using integer operations only (no FP64-pipe conversion)
-__device__ __forceinline__ int floor_nonneg(double T) {
-  const long long b = __double_as_longlong(T);
-  const int e = (int)((b >> 52) & 0x7ff) - 1023;
-  if (e < 0) return 0;
-  const long long m = (b & 0xfffffffffffffLL) | 0x10000000000000LL;
-  return (int)(m >> (52 - e));
-}
-
-// Prepare the table lookup for one T: ti >= 0 selects interval ti (of width 1/RYS_SUB),
-// else the large-T limit.
-__device__ __forceinline__ void rys_locate(double T, double tcut, int& ti, double& x, double& invT, double& rsqT) {
-  if (T < tcut) {
-    ti = floor_nonneg((double)RYS_SUB * T);
-    x = fma(2.0 * RYS_SUB, T, -(double)(2 * ti + 1));
-    invT = 0.0;
-    rsqT = 0.0;
+    for (int k = 0; k < (RYS_DEG + 1) / 2; ++k) {
+      const longlong2 v = __ldg(c + k);
+      row[2 * k] = v.x;
+      row[2 * k + 1] = v.y;
+    }
+    const int64_t fu = rys_fx_horner(row, at.x0, at.x1, &E);
+    u = rys_value(fu, E, R());
+#pragma unroll
+    for (int k = 0; k < (RYS_DEG + 1) / 2; ++k) {
+      const longlong2 v = __ldg(c + (RYS_DEG + 1) / 2 + k);
+      row[2 * k] = v.x;
+      row[2 * k + 1] = v.y;
+    }
+    const int64_t fw = rys_fx_horner(row, at.x0, at.x1, &E);
+    w = rys_value(fw, E, R());
   } else {
-    ti = -1;
-    x = 0.0;
-    invT = 1.0 / T;
-    rsqT = rsqrt(T);
+    u = (R)(__ldg(au + n) * at.rsqT * at.rsqT);
+    w = (R)(__ldg(aw + n) * at.rsqT);
   }
 }
 
-__device__ __forceinline__ void rys_root(const double* __restrict__ coef, const double* __restrict__ au,
-                                         const double* __restrict__ aw, int N, int ti, double x,
-                                         double invT, double rsqT, int n, double& u, double& w) {
-  if (ti >= 0) {
-    const double* c = coef + ((size_t)ti * N + n) * (2 * (RYS_DEG + 1));
-    u = horner_rys(c, x);
-    w = horner_rys(c + RYS_DEG + 1, x);
+// The same root and weight by Horner's rule in FP64, for kernels whose integer pipes are the busier
+// ones (eri_fixed.cu: (dp|pp) 54 ms against 61 ms with the fixed-point sums on the 16-atom build).
+__device__ __forceinline__ void rys_root64(const double* __restrict__ coef, const double* __restrict__ au,
+                                           const double* __restrict__ aw, int N, const RysAt& at, int n, double& u,
+                                           double& w) {
+  if (at.ti >= 0) {
+    const double2* c = reinterpret_cast<const double2*>(coef) + ((size_t)at.ti * N + n) * (RYS_DEG + 1);
+    // x from its halves, exactly rounded: x0 2^-31 + x1 2^-60
+    const double x = fma((double)at.x0, 1.0 / 2147483648.0, (double)at.x1 * (1.0 / 1152921504606846976.0));
+    double v[2];
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      double2 d = __ldg(c + p * (RYS_DEG + 1) / 2);
+      double a = fma(d.x, x, d.y);
+#pragma unroll
+      for (int k = 1; k < (RYS_DEG + 1) / 2; ++k) {
+        d = __ldg(c + p * (RYS_DEG + 1) / 2 + k);
+        a = fma(fma(a, x, d.x), x, d.y);
+      }
+      v[p] = a;
+    }
+    u = v[0];
+    w = v[1];
   } else {
-    u = __ldg(au + n) * invT;
-    w = __ldg(aw + n) * rsqT;
+    u = __ldg(au + n) * at.rsqT * at.rsqT;
+    w = __ldg(aw + n) * at.rsqT;
   }
+}
+
+// The lookup in a team's shared region (NPD doubles per primitive quartet, from entry o).
+__device__ __forceinline__ void rys_put_team(const Smem<double>& sd, int o, const RysAt& at) {
+  sd[o] = __hiloint2double(at.x0, (int)at.x1);
+  sd[o + 1] = at.rsqT;
+  sd[o + 2] = __hiloint2double(0, at.ti);
+}
+__device__ __forceinline__ RysAt rys_get_team(const Smem<double>& sd, int o) {
+  RysAt r;
+  r.x0 = __double2hiint(sd[o]);
+  r.x1 = (uint32_t)__double2loint(sd[o]);
+  r.rsqT = sd[o + 1];
+  r.ti = __double2loint(sd[o + 2]);
+  return r;
 }
 
 // ------------------------------------------------------------------ 2D recurrences
@@ -517,10 +577,11 @@ struct TaskCtx {
   const ShellPair* pairs;
   const PrimPair* prims;
   const PrimPairF* primsf;
+  const PrimFx* prfx;
   const double* D;
   double* J;
   double* K;
-  int nbf, nD, want;
+  int nbf, nD, want, pu;
 };
 
 __device__ __forceinline__ TaskCtx single_ctx(const KernelArgs& a) {
@@ -528,6 +589,8 @@ __device__ __forceinline__ TaskCtx single_ctx(const KernelArgs& a) {
   c.pairs = a.pairs;
   c.prims = a.prims;
   c.primsf = a.primsf;
+  c.prfx = a.prfx;
+  c.pu = a.pu;
   c.D = a.D;
   c.J = a.J;
   c.K = a.K;
@@ -535,6 +598,27 @@ __device__ __forceinline__ TaskCtx single_ctx(const KernelArgs& a) {
   c.nD = a.nD;
   c.want = a.want;
   return c;
+}
+
+// P - Q of primitive pairs x and y (indices ix, iy): from the integer positions, whose difference is
+// exact (rounding P itself costs 2^-53 |P| bohr, which tight shells see as sqrt(zeta) times that), or
+// from the doubles when the plan has none (pu < 0).
+__device__ __forceinline__ void pair_distance(const TaskCtx& tc, const PrimPair* x, const PrimPair* y, int ix, int iy,
+                                              double& d0, double& d1, double& d2) {
+  if (tc.pu >= 0) {
+    const longlong2* p = reinterpret_cast<const longlong2*>(tc.prfx + ix);
+    const longlong2* q = reinterpret_cast<const longlong2*>(tc.prfx + iy);
+    const longlong2 p0 = __ldg(p), q0 = __ldg(q);
+    const long long p2 = __ldg(reinterpret_cast<const long long*>(p + 1)), q2 = __ldg(reinterpret_cast<const long long*>(q + 1));
+    const double unit = __hiloint2double((1023 - tc.pu) << 20, 0);
+    d0 = unit * __ll2double_rn(p0.x - q0.x);
+    d1 = unit * __ll2double_rn(p0.y - q0.y);
+    d2 = unit * __ll2double_rn(p2 - q2);
+  } else {
+    d0 = x->P[0] - y->P[0];
+    d1 = x->P[1] - y->P[1];
+    d2 = x->P[2] - y->P[2];
+  }
 }
 
 // Resolve list position `task` of a JK launch into (bra pair, ket pair) and its job context.
@@ -547,6 +631,8 @@ __device__ __forceinline__ void resolve_task(const KernelArgs& a, long long task
     ctx.pairs = jd.pairs;
     ctx.prims = jd.prims;
     ctx.primsf = jd.primsf;
+    ctx.prfx = jd.prfx;
+    ctx.pu = jd.pu;
     ctx.D = jd.D;
     ctx.J = jd.J;
     ctx.K = jd.K;
@@ -584,7 +670,7 @@ __device__ __forceinline__ int quartet_category(const KernelArgs& a, const Shell
 
 // Per-primitive-quartet scalars in shared memory: NPD doubles (root lookup, FP64 always)
 // followed by NPR values of the recurrence type R.
-#define NPD 4
+#define NPD 3
 #define NPR 18
 
 template <typename R> struct PairOf;

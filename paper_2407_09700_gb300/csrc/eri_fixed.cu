@@ -100,21 +100,18 @@ __global__ void __launch_bounds__(TPB, 3) eri_fixed_kernel(const KernelArgs a) {
       for (int j = tl; j < bp; j += TS) {
         if (j < nbt) {
           const int q = qlo + q0 + j;
-          const PrimPair* x = tc.prims + boff + q / npk;
-          const PrimPair* y = tc.prims + koff + q % npk;
+          // ket primitives up and down in turn, so that neighbours in a batch have like exponents
+          const int ibp = q / npk, r = q - ibp * npk;
+          const int ix = boff + ibp, iy = koff + ((ibp & 1) ? npk - 1 - r : r);
+          const PrimPair* x = tc.prims + ix;
+          const PrimPair* y = tc.prims + iy;
           const double zeta = x->zeta, eta = y->zeta;
           const double rd = rsqrt(zeta + eta);
-          const double PQ0 = x->P[0] - y->P[0], PQ1 = x->P[1] - y->P[1], PQ2 = x->P[2] - y->P[2];
+          double PQ0, PQ1, PQ2;
+          pair_distance(tc, x, y, ix, iy, PQ0, PQ1, PQ2);
           const double inv_s = rd * rd;
           const double T = zeta * eta * inv_s * fma(PQ0, PQ0, fma(PQ1, PQ1, PQ2 * PQ2));
-          int ti;
-          double xx, invT, rsqT;
-          rys_locate(T, a.rys_tcut_d, ti, xx, invT, rsqT);
-          const int od = j * NPD;
-          sd[od + 0] = xx;
-          sd[od + 1] = invT;
-          sd[od + 2] = rsqT;
-          sd[od + 3] = __longlong_as_double((long long)ti);
+          rys_put_team(sd, j * NPD, rys_locate(T, a.rys_tcut_hi));
           const double rz = eta * inv_s, re = zeta * inv_s;
           const int o = j * NPR;
           sr[o + 0] = x->PA[0]; sr[o + 1] = x->PA[1]; sr[o + 2] = x->PA[2];
@@ -135,10 +132,9 @@ __global__ void __launch_bounds__(TPB, 3) eri_fixed_kernel(const KernelArgs a) {
           const int jn = tk / 3, ax = tk - jn * 3;
           const int j = jn / N, n = jn - (jn / N) * N;
           if (j < nbt) {
-            const int od = j * NPD, o = j * NPR;
+            const int o = j * NPR;
             double u, w;
-            rys_root(a.rys_coef, a.rys_au, a.rys_aw, N, (int)__double_as_longlong(sd[od + 3]), sd[od + 0],
-                     sd[od + 1], sd[od + 2], n, u, w);
+            rys_root64(a.rys_coef64, a.rys_au, a.rys_aw, N, rys_get_team(sd, j * NPD), n, u, w);
             const double B00 = u * sr[o + 12];
             const double B10 = fma(-u, sr[o + 13], sr[o + 16]);
             const double B01 = fma(-u, sr[o + 14], sr[o + 17]);
@@ -152,10 +148,9 @@ __global__ void __launch_bounds__(TPB, 3) eri_fixed_kernel(const KernelArgs a) {
         for (int tk = tl; tk < bp * N; tk += TS) {
           const int j = tk / N, n = tk - (tk / N) * N;
           if (j < nbt) {
-            const int od = j * NPD, o = j * NPR;
+            const int o = j * NPR;
             double u, w;
-            rys_root(a.rys_coef, a.rys_au, a.rys_aw, N, (int)__double_as_longlong(sd[od + 3]), sd[od + 0],
-                     sd[od + 1], sd[od + 2], n, u, w);
+            rys_root64(a.rys_coef64, a.rys_au, a.rys_aw, N, rys_get_team(sd, j * NPD), n, u, w);
             const double B00 = u * sr[o + 12];
             const double B10 = fma(-u, sr[o + 13], sr[o + 16]);
             const double B01 = fma(-u, sr[o + 14], sr[o + 17]);
@@ -285,7 +280,7 @@ __global__ void __launch_bounds__(TPB, 3) eri_fixed_kernel(const KernelArgs a) {
 }
 
 // instantiated lanes per quartet and tiles per lane and pass
-#define FIXED_KERNELS(X) X(8, 2) X(8, 3) X(8, 4) X(16, 3) X(16, 4) X(16, 5) X(32, 3) X(32, 4)
+#define FIXED_KERNELS(X) X(16, 2) X(16, 3) X(32, 3)
 
 const void* fixed_ptr(int ts, int tiles) {
 #define FIXED_CASE(T, NT) \

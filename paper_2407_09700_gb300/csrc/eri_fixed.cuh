@@ -11,8 +11,10 @@
 // |I| 2^-K < 1.  An entry is two limbs, l0 2^-top + l1 2^-(top + 28), both with its sign: 56
 // fraction bits for I_x, 57 for I_y and I_z.  Before the scales are taken, the factor w Theta of
 // I_z is spread over the three axes by powers of two (fx_third), so that a tight primitive's
-// large prefactor does not meet a diffuse one's large I_x and I_y in the scales' product.  A product I_x I_y keeps 57 fraction bits (cut by a
-// floor); the limb products of its sum with I_z accumulate by weight in 64-bit integers, exactly
+// large prefactor does not meet a diffuse one's large I_x and I_y in the scales' product, and a
+// batch holds primitive pairs of neighbouring exponents (sorted in the plan, the ket's up and down
+// in turn): with p and d exponents from 0.1 to 400 the error against quadruple precision is
+// 3.5e-16 (3.6e-15 unsorted, 1.0e-13 without the spreading too, FP64 8.6e-16).  A product I_x I_y keeps 57 fraction bits; the limb products of its sum with I_z accumulate by weight in 64-bit integers, exactly
 // (at most FX_TERMS (primitive, root) terms per batch fit the headroom), and a batch's sum
 // returns to FP64 once, at scale 2^(K_x + K_y + K_z).
 //
@@ -29,6 +31,11 @@
 
 #define FX_TERMS 32      // most (primitive, root) terms accumulated between two returns to FP64
 #define FX_LMAX 8        // most angular momentum la + lb + lc + ld of a class
+// Most binades (l0 + l1) / 2 log2(zeta ratio) over a pair's primitives: an entry of degree n scales
+// like zeta^(-n/2).  6-31G(d)-like shells have 13 and p, d exponents 0.1 .. 400 18 (no larger
+// error than FP64); at 30 (0.1 .. 4000 in p and d) the error is 5e-15 against 0.5e-15, so wider
+// shells keep FP64.
+#define FX_SPREAD 20.0
 #define FX_LIMB 28
 #define FX_MASK 0x0fffffff
 #define FX_POISON (1 << 20)   // K of an entry that held an infinity or a NaN
@@ -36,7 +43,7 @@
 // Fraction bits of l0: axis 0, 1, 2 = x, y, z.
 __host__ __device__ constexpr int fx_top(int ax) { return ax == 0 ? 28 : 29; }
 
-// floor(e / 3) for |e| <= 1100.
+// About e / 3 (any integer serves).
 __host__ __device__ __forceinline__ int fx_third(int e) { return (e * 21846) >> 16; }
 
 // Limbs of the double with words (hi, lo) at the scale of biased exponent emax >= its own,
@@ -51,9 +58,9 @@ __host__ __device__ __forceinline__ void fx_split(uint32_t hi, uint32_t lo, int 
   l[1] = ((int32_t)((uint32_t)t & FX_MASK) ^ s) - s;
 }
 
-// v = x y (floor; v[1] >= 0).
+// v = x y (to nearest; v[1] >= 0).
 __host__ __device__ __forceinline__ void fx_mul(const int32_t x[2], const int32_t y[2], int32_t v[2]) {
-  const int64_t d1 = (int64_t)x[0] * y[1] + (int64_t)x[1] * y[0];
+  const int64_t d1 = (int64_t)x[0] * y[1] + (1 << (FX_LIMB - 1)) + (int64_t)x[1] * y[0];
   const int64_t d0 = (int64_t)x[0] * y[0] + (d1 >> FX_LIMB);
   v[1] = (int32_t)((uint32_t)d0 & FX_MASK);
   v[0] = (int32_t)(d0 >> FX_LIMB);

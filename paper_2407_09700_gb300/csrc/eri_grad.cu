@@ -142,6 +142,7 @@ __global__ void __launch_bounds__(TPB, (TS == 1 ? 3 : 2)) eri_grad_kernel(const 
   extern __shared__ double smem[];
   const KernelArgs& a = ga.k;
   const GradDesc& g = ga.g;
+  const TaskCtx tc = single_ctx(a);
   // TS = TPB: one team per block (team barriers are __syncthreads), as in the J/K kernel
   constexpr bool BLK = TS > 32;
   static_assert(!BLK || TS == TPB, "a team is a warp's part or the whole block");
@@ -267,21 +268,16 @@ __global__ void __launch_bounds__(TPB, (TS == 1 ? 3 : 2)) eri_grad_kernel(const 
       for (int j = tl; j < bp; j += TS) {
         if (j < nbt) {
           const int q = q0 + j;
-          const PrimPair* x = a.prims + boff + q / npk;
-          const PrimPair* y = a.prims + koff + q % npk;
+          const int ix = boff + q / npk, iy = koff + q % npk;
+          const PrimPair* x = a.prims + ix;
+          const PrimPair* y = a.prims + iy;
           const double zeta = x->zeta, eta = y->zeta;
           const double rd = rsqrt(zeta + eta);
-          const double PQ0 = x->P[0] - y->P[0], PQ1 = x->P[1] - y->P[1], PQ2 = x->P[2] - y->P[2];
+          double PQ0, PQ1, PQ2;
+          pair_distance(tc, x, y, ix, iy, PQ0, PQ1, PQ2);
           const double inv_s = rd * rd;
           const double T = zeta * eta * inv_s * fma(PQ0, PQ0, fma(PQ1, PQ1, PQ2 * PQ2));
-          int ti;
-          double xx, invT, rsqT;
-          rys_locate(T, a.rys_tcut_d, ti, xx, invT, rsqT);
-          const int od = j * NPD;
-          sd[od + 0] = xx;
-          sd[od + 1] = invT;
-          sd[od + 2] = rsqT;
-          sd[od + 3] = __longlong_as_double((long long)ti);
+          rys_put_team(sd, j * NPD, rys_locate(T, a.rys_tcut_hi));
           const double rz = eta * inv_s, re = zeta * inv_s;
           const int o = j * GNPR;
           sr[o + 0] = x->PA[0]; sr[o + 1] = x->PA[1]; sr[o + 2] = x->PA[2];
@@ -307,10 +303,9 @@ __global__ void __launch_bounds__(TPB, (TS == 1 ? 3 : 2)) eri_grad_kernel(const 
           const int jn = tk / 3, ax = tk - jn * 3;
           const int j = jn / N, n = jn - (jn / N) * N;
           if (j < nbt) {
-            const int od = j * NPD, o = j * GNPR;
+            const int o = j * GNPR;
             double u, w;
-            rys_root(a.rys_coef, a.rys_au, a.rys_aw, N, (int)__double_as_longlong(sd[od + 3]), sd[od + 0],
-                     sd[od + 1], sd[od + 2], n, u, w);
+            rys_root(a.rys_coef, a.rys_au, a.rys_aw, N, rys_get_team(sd, j * NPD), n, u, w);
             const double B00 = u * sr[o + 12];
             const double B10 = fma(-u, sr[o + 13], sr[o + 16]);
             const double B01 = fma(-u, sr[o + 14], sr[o + 17]);
@@ -334,10 +329,9 @@ __global__ void __launch_bounds__(TPB, (TS == 1 ? 3 : 2)) eri_grad_kernel(const 
         for (int tk = tl; tk < bp * N; tk += TS) {
           const int j = tk / N, n = tk - (tk / N) * N;
           if (j < nbt) {
-            const int od = j * NPD, o = j * GNPR;
+            const int o = j * GNPR;
             double u, w;
-            rys_root(a.rys_coef, a.rys_au, a.rys_aw, N, (int)__double_as_longlong(sd[od + 3]), sd[od + 0],
-                     sd[od + 1], sd[od + 2], n, u, w);
+            rys_root(a.rys_coef, a.rys_au, a.rys_aw, N, rys_get_team(sd, j * NPD), n, u, w);
             const double B00 = u * sr[o + 12];
             const double B10 = fma(-u, sr[o + 13], sr[o + 16]);
             const double B01 = fma(-u, sr[o + 14], sr[o + 17]);

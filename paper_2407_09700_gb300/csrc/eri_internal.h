@@ -29,6 +29,22 @@ struct PrimPairF {
   float pad[2];
 };
 
+// The same primitive pair for the one-lane kernels' integer scalars (eri_scalar.cuh).  112 bytes,
+// 16-byte aligned.
+struct PrimFx {
+  int64_t P[3];    // P from the plan's origin, units of 2^-pu
+  int64_t Hm;      // 1 / zeta = Hm 2^(He - 62)
+  int64_t hz;      // 1 / (2 zeta) 2^-2a, units of 2^-60
+  int64_t PA[3];   // (P - A) 2^-a, units of 2^-60
+  double H;        // 1 / zeta
+  double E;        // PrimPair's E / sqrt(zeta)
+  int He;
+  int a;           // 2^a bounds every C of the pair (eri_scalar.cuh)
+  int64_t Sm;      // 1 / sqrt(zeta) = Sm 2^(Se - 62)
+  int Se;
+  int pad[3];
+};
+
 // One shell pair in canonical orientation (l of sh0 >= l of sh1).  64 bytes.
 struct ShellPair {
   int sh0, sh1;    // shell indices
@@ -106,7 +122,8 @@ struct JobDesc {
   const double* D;
   double* J;
   double* K;
-  int nbf, nD, want, pad;
+  const struct PrimFx* prfx;
+  int nbf, nD, want, pu;
   int type_off[ERI_NPAIRTYPE];
   int type_cnt[ERI_NPAIRTYPE];
 };
@@ -116,6 +133,8 @@ struct KernelArgs {
   const ShellPair* pairs;
   const PrimPair* prims;
   const PrimPairF* primsf;     // FP32 shadow (FP32 kernels)
+  const PrimFx* prfx;          // integer scalars of the one-lane kernels
+  int pu;                      // unit 2^-pu of PrimFx::P; < 0: the plan has no integer scalars
   // task space: bra pairs [bra0, bra0+nbra), ket pairs [ket0, ket0+nket); tri = same range, ket <= bra
   int bra0, nbra, ket0, nket, tri;
   long long ntask;
@@ -159,11 +178,13 @@ struct KernelArgs {
   unsigned long long* stats;   // [0] quartets computed, [1] primitive quartets
   unsigned* err;               // set to 1 when a bounded device wait gave up (staged kernels)
   // Rys table for this class's root count
-  const double* rys_coef;      // block of this N
+  const int64_t* rys_coef;     // block of this N: fixed-point rows (rys_fixed.h)
+  const double* rys_coef64;    // the same block as doubles (rys_table.h)
   const double* rys_au;
   const double* rys_aw;
-  int rys_tcut;
-  double rys_tcut_d;           // the same cutoff as a double
+  int rys_tcut_hi;             // high word of the large-T cutoff as a double
+  long long rys_tcut4;         // RYS_SUB times the cutoff, units of 2^-54
+  const void* rys_asym;        // per root: the limit's u T and w sqrt(T) as (mantissa, exponent)
 };
 
 // One angular-momentum class of the two-electron energy gradient (Sec. 4, Eqs. 11-14).
@@ -228,14 +249,17 @@ int erik_launch_dmax(const double* D, int nD, int nbf, int nsh, const int* sh_bf
                      double* Dmax, void* stream);
 int erik_launch_symmetrize(double* M, int nD, int nbf, void* stream);
 int erik_launch_symcheck(const double* D, int nD, int nbf, unsigned long long* out, void* stream);
-int erik_launch_rys(int N, int n, const double* T, double* u, double* w, const double* coef,
-                    const double* au, const double* aw, int tcut, void* stream);
+int erik_launch_rys(int N, int n, const double* T, double* u, double* w, const int64_t* coef,
+                    const double* au, const double* aw, int tcut_hi, void* stream);
 int erik_probe_fma(double* fp64_tflops, double* fp32_tflops);
 // compile-time specialised kernels of the small classes (eri_small.cu)
 int erik_upload_cart_tables_small(void);
 int erik_small_available(int la, int lb, int lc, int ld, int fp32);
 int erik_small_blocks_per_sm(int la, int lb, int lc, int ld, int fp32, int* out);
 int erik_launch_small(int la, int lb, int lc, int ld, int fp32, const struct KernelArgs* a, int grid, void* stream);
+// the FP64 launches of these classes in integer arithmetic
+int erik_small_fx_blocks_per_sm(int la, int lb, int lc, int ld, int* out);
+int erik_launch_small_fx(int la, int lb, int lc, int ld, const struct KernelArgs* a, int grid, void* stream);
 // class kernels with the fixed-point assembly (eri_fixed.cu): instantiated lanes per quartet and
 // tiles per lane and pass
 int erik_upload_cart_tables_fixed(void);

@@ -232,14 +232,12 @@ __global__ void symmetrize_kernel(double* M, int nD, int nbf) {
   }
 }
 
-__global__ void rys_test_kernel(int N, int n, const double* T, double* u, double* w, const double* coef,
-                                const double* au, const double* aw, int tcut) {
+__global__ void rys_test_kernel(int N, int n, const double* T, double* u, double* w, const int64_t* coef,
+                                const double* au, const double* aw, int tcut_hi) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
-  int ti;
-  double x, invT, rsqT;
-  rys_locate(T[t], tcut, ti, x, invT, rsqT);
-  for (int r = 0; r < N; ++r) rys_root(coef, au, aw, N, ti, x, invT, rsqT, r, u[t * N + r], w[t * N + r]);
+  const RysAt at = rys_locate(T[t], tcut_hi);
+  for (int r = 0; r < N; ++r) rys_root(coef, au, aw, N, at, r, u[t * N + r], w[t * N + r]);
 }
 
 template <typename Tp>
@@ -380,9 +378,9 @@ extern "C" int erik_launch_symmetrize(double* M, int nD, int nbf, void* stream) 
   return (int)cudaGetLastError();
 }
 
-extern "C" int erik_launch_rys(int N, int n, const double* T, double* u, double* w, const double* coef,
-                               const double* au, const double* aw, int tcut, void* stream) {
-  rys_test_kernel<<<(n + 127) / 128, 128, 0, (cudaStream_t)stream>>>(N, n, T, u, w, coef, au, aw, tcut);
+extern "C" int erik_launch_rys(int N, int n, const double* T, double* u, double* w, const int64_t* coef,
+                               const double* au, const double* aw, int tcut_hi, void* stream) {
+  rys_test_kernel<<<(n + 127) / 128, 128, 0, (cudaStream_t)stream>>>(N, n, T, u, w, coef, au, aw, tcut_hi);
   return (int)cudaGetLastError();
 }
 

@@ -25,7 +25,8 @@
 #include "../../include/eri.h"
 #include "eri_fixed.cuh"
 #include "eri_internal.h"
-#include "rys_table.h"
+#include "eri_scalar.cuh"
+#include "rys_fixed.h"
 
 namespace {
 
@@ -85,9 +86,11 @@ const CartTab& cart() {
 // ---------------------------------------------------------------- per-device shared state
 struct DeviceState {
   bool ready = false;
-  double* rys_coef = nullptr;
+  int64_t* rys_coef = nullptr;       // fixed-point rows (rys_fixed.h)
+  double* rys_coef64 = nullptr;      // as doubles
   double* rys_au = nullptr;
   double* rys_aw = nullptr;
+  int64_t* rys_asym = nullptr;       // [root][2][2]: u T and w sqrt(T) as (mantissa, exponent)
   uint32_t* outidx = nullptr;        // all 225 class index tables
   ClassDesc classes[ERI_NPAIRTYPE][ERI_NPAIRTYPE];
   int ts[ERI_NPAIRTYPE][ERI_NPAIRTYPE];
@@ -359,14 +362,14 @@ void make_class(int la, int lb, int lc, int ld, ClassDesc* c, int* ts, std::vect
     c->gmask_off = (int)idx->size();
     idx->insert(idx->end(), gm.begin(), gm.end());
   }
-  // per primitive quartet: 4 doubles (table lookup) + 18 recurrence-type scalars + three 2D tables
+  // per primitive quartet: 3 doubles (table lookup) + 18 recurrence-type scalars + three 2D tables
   // the tables of one (primitive, root, axis) lie nIs apart, odd in team kernels: the lanes
   // of a team building different tables then write distinct banks
   c->nIs = (T > 1) ? (c->nI | 1) : c->nI;
-  const int per_prim = 4 + 18 + 3 * c->nroots * c->nIs;
+  const int per_prim = 3 + 18 + 3 * c->nroots * c->nIs;
   c->bp = (T == 1) ? 1 : std::max(1, std::min(32, team_budget(T) / per_prim));
   c->team_doubles = team_stride(c->bp * per_prim, T, false);
-  c->team_doubles_f32 = team_stride(c->bp * 4 + (c->bp * (18 + 3 * c->nroots * c->nIs) + 1) / 2, T, true);
+  c->team_doubles_f32 = team_stride(c->bp * 3 + (c->bp * (18 + 3 * c->nroots * c->nIs) + 1) / 2, T, true);
   c->split3 = choose_split3(T, c->bp, c->nroots, c->nI, 0);
 
   // ---- shared products path (FP64 launches of the classes where it measured faster):
@@ -505,18 +508,14 @@ void make_fixed_class(int la, int lb, int lc, int ld, ClassDesc* c, int* ts, std
     z[v] = (uint32_t)(ct.lz[e] * L1 + ct.lz[f]);
   }
   std::vector<Tile> tiles = make_tiles(xy, z);
-  // the instantiation that runs the fewest tiles, padding included; of equal ones the larger
-  // team (longer batches)
-  long long best = -1;
-  for (int i = 0, t, nt; erik_fixed_variant(i, &t, &nt); ++i) {
-    const long long np = ((long long)tiles.size() + t * nt - 1) / (t * nt), run = np * t * nt;
-    if (best < 0 || run < best || (run == best && t > *ts)) {
-      best = run;
-      *ts = t;
-      c->tiles = nt;
-      c->npass = (int)np;
-    }
-  }
+  // 16 lanes while one pass of three tiles a lane holds the class, else a whole warp: a larger
+  // team's longer batches fill the root phase and return fewer sums to FP64 (16-atom medium build,
+  // against 8 lanes with the fewest padded tiles: (dp|dp) 50.2 -> 47.9 ms, (dp|ds) 70.5 -> 61.7)
+  const int nt0 = (int)tiles.size();
+  *ts = nt0 <= 48 ? 16 : 32;
+  c->tiles = nt0 <= 32 ? 2 : 3;
+  c->npass = (nt0 + *ts * c->tiles - 1) / (*ts * c->tiles);
+  const long long best = (long long)c->npass * *ts * c->tiles;
   const int T = *ts;
   c->xy = 0;
   c->stage = 0;
@@ -532,9 +531,9 @@ void make_fixed_class(int la, int lb, int lc, int ld, ClassDesc* c, int* ts, std
   for (const Tile& t : tiles) idx->insert(idx->end(), t.dst, t.dst + 4);
   c->gmask_off = 0;
   c->nIs = c->nI | 1;
-  // per primitive quartet 22 scalars and three tables per root, per team K of the 3 nI entries
+  // per primitive quartet 21 scalars and three tables per root, per team K of the 3 nI entries
   // and of the steps
-  const int per_prim = 4 + 18 + 3 * c->nroots * c->nIs, fixed = (3 * c->nI + FX_TERMS + 1) / 2;
+  const int per_prim = 3 + 18 + 3 * c->nroots * c->nIs, fixed = (3 * c->nI + FX_TERMS + 1) / 2;
   c->bp = std::max(1, std::min(FX_TERMS / c->nroots, (fixed_budget(T) - fixed) / per_prim));
   c->team_doubles = team_stride(c->bp * per_prim + fixed, T, false);
   c->team_doubles_xy = c->team_doubles_f32 = c->bp_xy = 0;
@@ -601,9 +600,9 @@ void make_grad_class(int la, int lb, int lc, int ld, GradDesc* g, int* ts, std::
   idx->insert(idx->end(), dst.begin(), dst.end());
   g->gmask_off = (int)idx->size();
   idx->insert(idx->end(), gm.begin(), gm.end());
-  // per primitive quartet: 4 doubles (table lookup) + 21 scalars + the I_x, I_y tables and
+  // per primitive quartet: 3 doubles (table lookup) + 21 scalars + the I_x, I_y tables and
   // four weighted I_z tables (weights 1, 2 alpha, 2 beta, 2 gamma)
-  const int per_prim = 4 + 21 + 6 * NnI;
+  const int per_prim = 3 + 21 + 6 * NnI;
   if (*ts == 1) {
     g->bp = 1;
   } else {
@@ -648,12 +647,26 @@ eri_status device_init(int dev, DeviceState** out) {
     CUDA_TRY(erik_upload_cart_tables_fixed());
     CUDA_TRY(erik_class_spec_prepare());
     size_t ncoef = (size_t)RYS_NCOEF, nas = (size_t)RYS_ASYM_OFFSET[RYS_NMAX] + RYS_NMAX;
-    CUDA_TRY(cudaMalloc(&s.rys_coef, sizeof(double) * ncoef));
+    std::vector<int64_t> rows(ncoef);
+    for (size_t k = 0; k < ncoef; k += RYS_DEG + 1) rys_fx_row(RYS_COEF + k, &rows[k]);
+    CUDA_TRY(cudaMalloc(&s.rys_coef, sizeof(int64_t) * ncoef));
+    CUDA_TRY(cudaMalloc(&s.rys_coef64, sizeof(double) * ncoef));
+    CUDA_TRY(cudaMemcpy(s.rys_coef64, RYS_COEF, sizeof(double) * ncoef, cudaMemcpyHostToDevice));
     CUDA_TRY(cudaMalloc(&s.rys_au, sizeof(double) * nas));
     CUDA_TRY(cudaMalloc(&s.rys_aw, sizeof(double) * nas));
-    CUDA_TRY(cudaMemcpy(s.rys_coef, RYS_COEF, sizeof(double) * ncoef, cudaMemcpyHostToDevice));
+    CUDA_TRY(cudaMemcpy(s.rys_coef, rows.data(), sizeof(int64_t) * ncoef, cudaMemcpyHostToDevice));
     CUDA_TRY(cudaMemcpy(s.rys_au, RYS_ASYM_U, sizeof(double) * nas, cudaMemcpyHostToDevice));
     CUDA_TRY(cudaMemcpy(s.rys_aw, RYS_ASYM_W, sizeof(double) * nas, cudaMemcpyHostToDevice));
+    std::vector<int64_t> asym(4 * nas);
+    for (size_t k = 0; k < nas; ++k)
+      for (int i = 0; i < 2; ++i) {
+        int e = 0;
+        const double v = i ? RYS_ASYM_W[k] : RYS_ASYM_U[k];
+        if (v > 0) sx_from_double(v, &asym[4 * k + 2 * i], &e);
+        asym[4 * k + 2 * i + 1] = e;
+      }
+    CUDA_TRY(cudaMalloc(&s.rys_asym, sizeof(int64_t) * asym.size()));
+    CUDA_TRY(cudaMemcpy(s.rys_asym, asym.data(), sizeof(int64_t) * asym.size(), cudaMemcpyHostToDevice));
     std::vector<uint32_t> all, one;
     size_t offs[ERI_NPAIRTYPE][ERI_NPAIRTYPE], foffs[ERI_NPAIRTYPE][ERI_NPAIRTYPE];
     for (int X = 0; X < ERI_NPAIRTYPE; ++X)
@@ -802,6 +815,7 @@ struct eri_plan {
   // kept pairs (Q > tau)
   int type_off[ERI_NPAIRTYPE] = {0}, type_cnt[ERI_NPAIRTYPE] = {0};
   int type_maxprim[ERI_NPAIRTYPE] = {0};   // most primitive pairs of a kept pair, per type
+  double type_spread[ERI_NPAIRTYPE] = {0}; // (l0 + l1) / 2 log2 of the largest ratio of a kept pair's zeta
   int npairs_kept = 0;
   std::vector<double> Q;             // [nshell*nshell]
   std::vector<double> Qe;            // [nshell*nshell] transfer-aware factors of the mixed split
@@ -810,6 +824,9 @@ struct eri_plan {
   ShellPair* d_pairs = nullptr;
   PrimPair* d_prims = nullptr;
   PrimPairF* d_primsf = nullptr;
+  PrimFx* d_prfx = nullptr;
+  int pu = -1;                       // unit 2^-pu of PrimFx::P (< 0: no integer positions)
+  bool fx_ok = true;                 // every exponent within the integer scalars' range
   int* d_sh_bf0 = nullptr;
   int* d_sh_n = nullptr;
   int* d_sh_atom = nullptr;
@@ -905,6 +922,13 @@ eri_status launch_shape(eri_plan* p, int X, int Y, int fp32, int fixed, long lon
   return ERI_OK;
 }
 
+int rys_tcut_hi(int N) {
+  const double t = (double)RYS_TCUT[N];
+  uint64_t u;
+  memcpy(&u, &t, sizeof(u));
+  return (int)(u >> 32);
+}
+
 KernelArgs base_args(eri_plan* p, int X, int Y) {
   KernelArgs a;
   memset(&a, 0, sizeof(a));
@@ -915,10 +939,14 @@ KernelArgs base_args(eri_plan* p, int X, int Y) {
   a.nbf = p->nbf;
   const int N = a.c.nroots;
   a.rys_coef = p->dev->rys_coef + RYS_COEF_OFFSET[N];
+  a.rys_coef64 = p->dev->rys_coef64 + RYS_COEF_OFFSET[N];
   a.rys_au = p->dev->rys_au + RYS_ASYM_OFFSET[N];
   a.rys_aw = p->dev->rys_aw + RYS_ASYM_OFFSET[N];
-  a.rys_tcut = RYS_TCUT[N];
-  a.rys_tcut_d = (double)RYS_TCUT[N];
+  a.rys_tcut_hi = rys_tcut_hi(N);
+  a.rys_tcut4 = (long long)(RYS_SUB * RYS_TCUT[N]) << 54;
+  a.rys_asym = p->dev->rys_asym + 4 * RYS_ASYM_OFFSET[N];
+  a.prfx = p->d_prfx;
+  a.pu = p->pu;
   a.err = p->d_err;
   return a;
 }
@@ -980,11 +1008,59 @@ eri_status validate_basis(const eri_basis* b) {
 }
 
 
+// Integer shadows of the primitive pairs (eri_scalar.cuh): positions from a point near the
+// molecule's middle in units of 2^-pu that hold every P - Q in 60 bits.
+void make_prim_fx(eri_plan* p, PrimFx* out) {
+  double lo[3], hi[3], mid[3], ext = 0.0;
+  for (int x = 0; x < 3; ++x) {
+    lo[x] = hi[x] = p->coords[x];
+    for (int k = 1; k < p->natm; ++k) {
+      lo[x] = std::min(lo[x], p->coords[3 * k + x]);
+      hi[x] = std::max(hi[x], p->coords[3 * k + x]);
+    }
+    mid[x] = std::nearbyint(0.5 * (lo[x] + hi[x]));
+    ext = std::max(ext, std::max(hi[x] - mid[x], mid[x] - lo[x]));
+  }
+  int e = 0;
+  (void)std::frexp(2.0 * ext, &e);                       // |P - Q| <= 2 ext < 2^e
+  p->pu = 59 - e;
+  p->fx_ok = e < 59;
+  const double upu = p->fx_ok ? sx_pow2(p->pu) : 0.0;
+  std::vector<int64_t> org(3 * p->natm, 0);
+  if (p->fx_ok)
+    for (int k = 0; k < 3 * p->natm; ++k) org[k] = std::llrint((p->coords[k] - mid[k % 3]) * upu);
+  for (const ShellPair& sp : p->pairs_all)
+    for (int k = sp.prim_off; k < sp.prim_off + sp.nprim; ++k) {
+      const PrimPair& q = p->prims[k];
+      PrimFx& f = out[k];
+      memset(&f, 0, sizeof(f));
+      if (!(q.zeta > 1e-30 && q.zeta < 1e30) || !std::isfinite(q.E)) {
+        p->fx_ok = false;
+        continue;
+      }
+      f.H = 2.0 * q.hz;
+      const double root = std::sqrt(f.H);
+      f.E = q.E * root;
+      sx_from_double(f.H, &f.Hm, &f.He);
+      sx_from_double(root, &f.Sm, &f.Se);
+      double pa = 0.0;
+      for (int x = 0; x < 3; ++x) pa = std::max(pa, std::fabs(q.PA[x]));
+      int64_t m;
+      sx_from_double(1.0001 * (pa + 2.3507 * root), &m, &f.a);
+      const double u60 = sx_pow2(60 - f.a);
+      f.hz = std::llrint(q.hz * u60 * sx_pow2(-f.a));
+      for (int x = 0; x < 3; ++x) {
+        f.PA[x] = std::llrint(q.PA[x] * u60);
+        if (p->fx_ok) f.P[x] = org[3 * p->sh_atom[sp.sh0] + x] + std::llrint(q.PA[x] * upu);
+      }
+    }
+}
+
 // ---------------------------------------------------------------- J/K launch machinery
 struct Launch {
   int X, Y, fp32, grid, smem, ts;
   long long nt;
-  int small;             // 1: compile-time specialised kernel (eri_small.cu)
+  int small;             // compile-time specialised kernel (eri_small.cu): 1 floating point, 2 integer
   int split;             // 1: the class runs an FP64 and an FP32 launch (mixed mode)
   int qsplit;            // tasks per quartet (ranges of its primitive quartets), 1 = none
   int fixed;             // 1: FP64 launch with the fixed-point assembly (eri_fixed.cu)
@@ -992,6 +1068,11 @@ struct Launch {
 
 const ClassDesc& launch_class(const eri_plan* p, const Launch& l) {
   return l.fixed ? p->dev->fclasses[l.X][l.Y] : p->dev->classes[l.X][l.Y];
+}
+
+// Scratch doubles of one block (the one-lane kernels need none).
+size_t block_scratch(const eri_plan* p, const Launch& l) {
+  return l.small ? 0 : (size_t)(128 / l.ts) * (size_t)launch_class(p, l).scratch_per_team;
 }
 
 // Classes with at most this many candidate quartets screen in the kernel instead of being
@@ -1014,22 +1095,26 @@ int choose_qsplit(long long nt, long long teams, int maxq, int minq) {
 
 // Kernel, split, grid and shared memory of a J/K launch over l->nt candidate quartets of at most
 // maxq primitive quartets: the specialised one-lane kernel where the class runs with one lane
-// per quartet (FP32: whenever one exists), else for FP64 the fixed-point assembly where the
+// per quartet (FP32: whenever one exists; FP64: in integers when fx_ok; spread: type_spread of the
+// class's wider type), else for FP64 the fixed-point assembly where the
 // class has one, else the FP64 / FP32 class kernel.
-eri_status shape_launch(eri_plan* p, int maxq, Launch* l) {
+eri_status shape_launch(eri_plan* p, int maxq, bool fx_ok, double spread, Launch* l) {
   const ClassDesc& cd = p->dev->classes[l->X][l->Y];
   if ((l->fp32 || p->dev->ts[l->X][l->Y] == 1) && erik_small_available(cd.la, cd.lb, cd.lc, cd.ld, l->fp32)) {
     int bps = 0;
-    CUDA_TRY(erik_small_blocks_per_sm(cd.la, cd.lb, cd.lc, cd.ld, l->fp32, &bps));
+    l->small = !l->fp32 && fx_ok ? 2 : 1;
+    if (l->small == 2)
+      CUDA_TRY(erik_small_fx_blocks_per_sm(cd.la, cd.lb, cd.lc, cd.ld, &bps));
+    else
+      CUDA_TRY(erik_small_blocks_per_sm(cd.la, cd.lb, cd.lc, cd.ld, l->fp32, &bps));
     const long long full = (long long)p->dev->sms * std::max(bps, 1);
     l->ts = 1;
     l->qsplit = choose_qsplit(l->nt, full * 128, maxq, 2);
     l->grid = (int)std::max(1LL, std::min(full, (l->nt * l->qsplit + 127) / 128));
     l->smem = 0;
-    l->small = 1;
     return ERI_OK;
   }
-  l->fixed = !l->fp32 && p->dev->fts[l->X][l->Y] > 0;
+  l->fixed = !l->fp32 && p->dev->fts[l->X][l->Y] > 0 && spread <= FX_SPREAD;
   const ClassDesc& c = launch_class(p, *l);
   // a full grid first: the teams it holds decide the split, the split the grid
   eri_status s = launch_shape(p, l->X, l->Y, l->fp32, l->fixed, 1LL << 40, &l->grid, &l->smem, &l->ts);
@@ -1041,6 +1126,7 @@ eri_status shape_launch(eri_plan* p, int maxq, Launch* l) {
 // Run the launch's kernel (a.c is set to its class).
 int run_launch(const eri_plan* p, const Launch& l, KernelArgs& a, cudaStream_t st) {
   a.c = launch_class(p, l);
+  if (l.small == 2) return erik_launch_small_fx(a.c.la, a.c.lb, a.c.lc, a.c.ld, &a, l.grid, st);
   if (l.small) return erik_launch_small(a.c.la, a.c.lb, a.c.lc, a.c.ld, l.fp32, &a, l.grid, st);
   if (l.fixed) return erik_launch_fixed(l.ts, a.c.tiles, &a, l.grid, l.smem, st);
   return erik_launch_class(l.ts, l.fp32, &a, l.grid, l.smem, st);
@@ -1059,11 +1145,12 @@ eri_status check_jk_args(eri_plan* p, const double* D, int nD, double* J, double
 
 // In the mixed mode, whether class (X|Y) gets an FP32 launch: its task space must reach the
 // plan's mixed_min_tasks (a second launch for a handful of quartets costs more than the FP32
-// arithmetic saves); otherwise every quartet of the class runs in FP64.
+// arithmetic saves), and the plan's exponents the integer scalars' range (far beyond FP32's);
+// otherwise every quartet of the class runs in FP64.
 bool fp32_pays(const eri_plan* p, int X, int Y, long long nt) {
   (void)X;
   (void)Y;
-  return nt >= (long long)p->opts.mixed_min_tasks;
+  return p->fx_ok && nt >= (long long)p->opts.mixed_min_tasks;
 }
 
 // One launch per class (pair-type pair X >= Y); in the mixed mode one FP64 and one FP32
@@ -1081,17 +1168,18 @@ eri_status plan_launches(eri_plan* p, size_t max_scratch, std::vector<Launch>* o
       const int np = (nprec == 2 && fp32_pays(p, X, Y, nt)) ? 2 : 1;
       for (int fp32 = 0; fp32 < np; ++fp32) {
         Launch l{X, Y, fp32, 0, 0, 0, nt, 0, np == 2 ? 1 : 0, 1, 0};
-        eri_status s = shape_launch(p, p->type_maxprim[X] * p->type_maxprim[Y], &l);
+        eri_status s = shape_launch(p, p->type_maxprim[X] * p->type_maxprim[Y], p->fx_ok,
+                                    std::max(p->type_spread[X], p->type_spread[Y]), &l);
         if (s != ERI_OK) return s;
         if (max_scratch > 0) {
           const ClassDesc& c = launch_class(p, l);
-          const size_t per_block = (size_t)(128 / l.ts) * (size_t)c.scratch_per_team;
+          const size_t per_block = block_scratch(p, l);
           if (per_block > max_scratch)
             return fail(ERI_ERR_ARG,
                         "class (%d%d|%d%d) needs %zu bytes of scratch for one block, more than the %zu-byte "
                         "static scratch of eri_jk_noalloc",
                         c.la, c.lb, c.lc, c.ld, per_block * sizeof(double), max_scratch * sizeof(double));
-          l.grid = (int)std::min<size_t>((size_t)l.grid, max_scratch / per_block);
+          if (per_block) l.grid = (int)std::min<size_t>((size_t)l.grid, max_scratch / per_block);
         }
         out->push_back(l);
       }
@@ -1200,7 +1288,7 @@ eri_status run_jk(eri_plan* p, const std::vector<Launch>& launches, const double
       p->last_launch_ts.push_back(l.ts);
       p->last_launch_grid.push_back(l.grid);
       p->last_launch_fp32.push_back(l.fp32);
-      p->last_launch_small.push_back(l.small);
+      p->last_launch_small.push_back(l.small ? 1 : 0);
       p->last_launch_fixed.push_back(l.fixed);
       p->last_launch_qsplit.push_back(l.qsplit);
       p->last_launch_listed.push_back(listed ? 1 : 0);
@@ -1232,7 +1320,7 @@ eri_status size_jk_buffers(eri_plan* p, std::vector<Launch>* launches, size_t* n
   if ((s = plan_launches(p, 0, launches)) != ERI_OK) return s;
   size_t need = 0;
   for (const Launch& l : *launches)
-    need = std::max(need, (size_t)l.grid * (size_t)(128 / l.ts) * (size_t)launch_class(p, l).scratch_per_team);
+    need = std::max(need, (size_t)l.grid * block_scratch(p, l));
   need = (need + 31) & ~(size_t)31;
   size_t maxnt = 1;
   for (const Launch& l : *launches)
@@ -1286,7 +1374,7 @@ eri_status eri_plan_destroy(eri_plan* p) {
   if (p->side) cudaStreamDestroy(p->side);
   if (p->ev_fork) cudaEventDestroy(p->ev_fork);
   if (p->ev_join) cudaEventDestroy(p->ev_join);
-  void* bufs[] = {p->d_pairs_all, p->d_pairs, p->d_prims, p->d_primsf, p->d_sh_bf0, p->d_sh_n, p->d_sh_atom, p->d_Dmax, p->d_counters,
+  void* bufs[] = {p->d_pairs_all, p->d_pairs, p->d_prims, p->d_primsf, p->d_prfx, p->d_sh_bf0, p->d_sh_n, p->d_sh_atom, p->d_Dmax, p->d_counters,
                   p->d_stats, p->d_scratch, p->d_tasks, p->d_out, p->d_off, p->d_host_io, p->d_tlist,
                   p->d_tcount, p->d_tiles, p->d_gstats, p->d_symchk, p->d_err};
   for (void* b : bufs)
@@ -1368,6 +1456,13 @@ eri_status eri_plan_create(const eri_basis* basis, const eri_opts* opts, void* c
           if (arg < best_arg) { best_arg = arg; best = code; }
         }
       if (t.keep.empty()) t.keep.push_back(best);
+      // by total exponent: the fixed-point kernels scale batches of neighbours together
+      std::stable_sort(t.keep.begin(), t.keep.end(), [&](int c0, int c1) {
+        const int nb = p->sh_nprim[b];
+        const double z0 = p->exps[p->sh_off[a] + c0 / nb] + p->exps[p->sh_off[b] + c0 % nb];
+        const double z1 = p->exps[p->sh_off[a] + c1 / nb] + p->exps[p->sh_off[b] + c1 % nb];
+        return z0 < z1;
+      });
       t.np = (int)t.keep.size();
       tmp.push_back(std::move(t));
     }
@@ -1403,7 +1498,7 @@ eri_status eri_plan_create(const eri_basis* basis, const eri_opts* opts, void* c
       pp.zeta = al + be;
       for (int x = 0; x < 3; ++x) {
         pp.P[x] = (al * A[x] + be * B[x]) / pp.zeta;
-        pp.PA[x] = pp.P[x] - A[x];
+        pp.PA[x] = -(be / pp.zeta) * sp.AB[x];   // P - A without the cancellation
       }
       pp.E = pref / pp.zeta * std::exp(-al * be / pp.zeta * AB2) * ca * cb;
       pp.hz = 0.5 / pp.zeta;
@@ -1423,6 +1518,7 @@ eri_status eri_plan_create(const eri_basis* basis, const eri_opts* opts, void* c
       cudaMalloc(&p->d_pairs, sizeof(ShellPair) * npair) != cudaSuccess ||
       cudaMalloc(&p->d_prims, sizeof(PrimPair) * p->prims.size()) != cudaSuccess ||
       cudaMalloc(&p->d_primsf, sizeof(PrimPairF) * p->prims.size()) != cudaSuccess ||
+      cudaMalloc(&p->d_prfx, sizeof(PrimFx) * p->prims.size()) != cudaSuccess ||
       cudaMalloc(&p->d_sh_bf0, sizeof(int) * p->nshell) != cudaSuccess ||
       cudaMalloc(&p->d_sh_n, sizeof(int) * p->nshell) != cudaSuccess ||
       cudaMalloc(&p->d_sh_atom, sizeof(int) * p->nshell) != cudaSuccess ||
@@ -1454,6 +1550,10 @@ eri_status eri_plan_create(const eri_basis* basis, const eri_opts* opts, void* c
     f.pad[0] = f.pad[1] = 0.f;
   }
   PLAN_TRY(cudaMemcpyAsync(p->d_primsf, primsf.data(), sizeof(PrimPairF) * primsf.size(), cudaMemcpyHostToDevice, st));
+  std::vector<PrimFx> prfx(p->prims.size());
+  make_prim_fx(p, prfx.data());
+  if (!p->fx_ok) p->pu = -1;
+  PLAN_TRY(cudaMemcpyAsync(p->d_prfx, prfx.data(), sizeof(PrimFx) * prfx.size(), cudaMemcpyHostToDevice, st));
   PLAN_TRY(cudaMemcpyAsync(p->d_sh_bf0, p->sh_bf0.data(), sizeof(int) * p->nshell, cudaMemcpyHostToDevice, st));
   PLAN_TRY(cudaMemcpyAsync(p->d_sh_n, sh_n.data(), sizeof(int) * p->nshell, cudaMemcpyHostToDevice, st));
   PLAN_TRY(cudaMemcpyAsync(p->d_sh_atom, p->sh_atom.data(), sizeof(int) * p->nshell, cudaMemcpyHostToDevice, st));
@@ -1501,6 +1601,12 @@ eri_status eri_plan_create(const eri_basis* basis, const eri_opts* opts, void* c
       if (sp.Q > p->opts.screen_thresh) {
         kept.push_back(sp);
         p->type_maxprim[X] = std::max(p->type_maxprim[X], sp.nprim);
+        double zlo = p->prims[sp.prim_off].zeta, zhi = zlo;
+        for (int q = 1; q < sp.nprim; ++q) {
+          zlo = std::min(zlo, p->prims[sp.prim_off + q].zeta);
+          zhi = std::max(zhi, p->prims[sp.prim_off + q].zeta);
+        }
+        p->type_spread[X] = std::max(p->type_spread[X], 0.5 * (p->sh_l[sp.sh0] + p->sh_l[sp.sh1]) * std::log2(zhi / zlo));
       }
     }
     p->type_cnt[X] = (int)kept.size() - p->type_off[X];
@@ -1597,8 +1703,7 @@ eri_status eri_jk_grad(eri_plan* p, const double* D, double* gJ, double* gK, voi
     a.rys_coef = p->dev->rys_coef + RYS_COEF_OFFSET[N];
     a.rys_au = p->dev->rys_au + RYS_ASYM_OFFSET[N];
     a.rys_aw = p->dev->rys_aw + RYS_ASYM_OFFSET[N];
-    a.rys_tcut = RYS_TCUT[N];
-    a.rys_tcut_d = (double)RYS_TCUT[N];
+    a.rys_tcut_hi = rys_tcut_hi(N);
     a.pairs = p->d_pairs;
     a.bra0 = p->type_off[l.X];
     a.nbra = p->type_cnt[l.X];
@@ -1752,7 +1857,7 @@ eri_status eri_rys_roots(int N, int n, const double* T, double* u, double* w) {
   cudaError_t e = cudaMemcpy(dT, T, sizeof(double) * n, cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
     e = (cudaError_t)erik_launch_rys(N, n, dT, du, dw, ds->rys_coef + RYS_COEF_OFFSET[N], ds->rys_au + RYS_ASYM_OFFSET[N],
-                                     ds->rys_aw + RYS_ASYM_OFFSET[N], RYS_TCUT[N], nullptr);
+                                     ds->rys_aw + RYS_ASYM_OFFSET[N], rys_tcut_hi(N), nullptr);
   if (e == cudaSuccess) e = cudaMemcpy(u, du, sizeof(double) * n * N, cudaMemcpyDeviceToHost);
   if (e == cudaSuccess) e = cudaMemcpy(w, dw, sizeof(double) * n * N, cudaMemcpyDeviceToHost);
   cudaFree(dT); cudaFree(du); cudaFree(dw);
@@ -1949,7 +2054,7 @@ eri_status eri_check_class_tables(int* nclasses, int* problems) {
             if (seen[v] != 1) ++bad;
           if (c.bp * c.nroots > FX_TERMS || 8L * c.team_doubles * (128 / ts) > 200 * 1024) ++bad;
           const int ntab = c.bp * 3 * c.nroots * c.nIs;
-          if (8L * c.team_doubles < 8L * c.bp * 22 + 8L * ntab + 4L * (3 * c.nI + c.bp * c.nroots)) ++bad;
+          if (8L * c.team_doubles < 8L * c.bp * 21 + 8L * ntab + 4L * (3 * c.nI + c.bp * c.nroots)) ++bad;
         }
       }
       {
@@ -2131,13 +2236,17 @@ eri_status eri_jk_batch(eri_batch* b, int njobs, eri_plan* const* plans, const d
   eri_plan* p0 = plans[0];
   // ---- job descriptors
   std::vector<JobDesc> jobs(njobs);
+  bool fx_ok = true;
   for (int j = 0; j < njobs; ++j) {
     eri_plan* p = plans[j];
+    fx_ok = fx_ok && p->fx_ok;
     JobDesc& jd = jobs[j];
     memset(&jd, 0, sizeof(jd));
     jd.pairs = p->d_pairs;
     jd.prims = p->d_prims;
     jd.primsf = p->d_primsf;
+    jd.prfx = p->d_prfx;
+    jd.pu = p->pu;
     jd.D = D[j];
     jd.J = J[j];
     jd.K = K[j];
@@ -2161,23 +2270,25 @@ eri_status eri_jk_batch(eri_batch* b, int njobs, eri_plan* const* plans, const d
   if ((s = ensure_batch_buf(b, &b->d_jobs, &b->jobs_cap, (size_t)njobs, st)) != ERI_OK) return s;
   CUDA_TRY(cudaMemcpyAsync(b->d_jobs, jobs.data(), sizeof(JobDesc) * njobs, cudaMemcpyHostToDevice, st));
   // ---- classes present in any job, their merged capacities and launch shapes
-  struct BL { int X, Y; long long total; long long maxnt; int any_fp32, maxq; };
+  struct BL { int X, Y; long long total; long long maxnt; int any_fp32, maxq; double spread; };
   std::vector<BL> cls;
   for (int X = 0; X < ERI_NPAIRTYPE; ++X)
     for (int Y = 0; Y <= X; ++Y) {
       long long tot = 0, mx = 0;
       int any32 = 0, maxq = 1;
+      double spread = 0.0;
       for (int j = 0; j < njobs; ++j) {
         const long long nx = plans[j]->type_cnt[X], ny = plans[j]->type_cnt[Y];
         if (!nx || !ny) continue;
         maxq = std::max(maxq, plans[j]->type_maxprim[X] * plans[j]->type_maxprim[Y]);
+        spread = std::max(spread, std::max(plans[j]->type_spread[X], plans[j]->type_spread[Y]));
         const long long nt = (X == Y) ? nx * (nx + 1) / 2 : nx * ny;
         if ((unsigned long long)nt > 0xffffffffULL) return fail(ERI_ERR_ARG, "job %d has more than 2^32 tasks in a class", j);
         tot += nt;
         mx = std::max(mx, nt);
         if (plans[j]->opts.precision == ERI_MIXED && fp32_pays(plans[j], X, Y, nt)) any32 = 1;
       }
-      if (tot) cls.push_back({X, Y, tot, mx, any32, maxq});
+      if (tot) cls.push_back({X, Y, tot, mx, any32, maxq, spread});
     }
   size_t cap = 1, tcap = 2, need = 0;
   std::vector<Launch> launches;
@@ -2187,8 +2298,8 @@ eri_status eri_jk_batch(eri_batch* b, int njobs, eri_plan* const* plans, const d
     for (int fp32 = 0; fp32 < (c.any_fp32 ? 2 : 1); ++fp32) {
       // as in eri_jk, over the jobs' merged quartets
       Launch l{c.X, c.Y, fp32, 0, 0, 0, c.total, 0, 0, 1, 0};
-      if ((s = shape_launch(p0, c.maxq, &l)) != ERI_OK) return s;
-      need = std::max(need, (size_t)l.grid * (size_t)(128 / l.ts) * (size_t)launch_class(p0, l).scratch_per_team);
+      if ((s = shape_launch(p0, c.maxq, fx_ok, c.spread, &l)) != ERI_OK) return s;
+      need = std::max(need, (size_t)l.grid * block_scratch(p0, l));
       launches.push_back(l);
     }
   }

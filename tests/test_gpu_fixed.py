@@ -1,5 +1,7 @@
-"""J/K of the classes with the fixed-point Eq. 1 assembly (s, p and d shells in more than one
-lane per quartet) against the oracle: batches of one primitive quartet, batches that do not
+"""J/K of the classes that run in integer arithmetic against the oracle.
+
+The classes with the fixed-point Eq. 1 assembly (s, p and d shells in more than one
+lane per quartet): batches of one primitive quartet, batches that do not
 divide the primitive quartets, and exponents over many binades (one scale per batch and table
 entry must hold tight and diffuse primitives together)."""
 
@@ -48,3 +50,47 @@ def test_jk_fixed_point_classes(depths, beta, spread):
     Jr, Kr, _ = oracle.jk(m, tau=0.0)
     for got, ref in ((J, Jr), (K, Kr)):
         assert np.abs(got.cpu().numpy() - ref).max() <= 1e-12 * np.abs(ref).max()
+
+
+def _check(m, tol=1e-12, plan=None):
+    plan = plan or pkg.Plan(m, tau=0.0)
+    J, K = plan.jk(torch.from_numpy(m.D).cuda())
+    Jr, Kr, _ = oracle.jk(m, tau=0.0)
+    for got, ref in ((J, Jr), (K, Kr)):
+        assert np.abs(got.cpu().numpy() - ref).max() <= tol * np.abs(ref).max()
+
+
+# The one-lane classes' integer scalars: one centre (P = Q, T = 0), the large-T limit (centres far
+# apart: every T above the table), extents that shift the unit of P, exponents over eight decades,
+# and an exponent outside the integers' range, which keeps FP64 kernels.  Tolerance as above.
+@pytest.mark.parametrize("dist,exps", [
+    (0.0, (0.2, 1.1)),
+    (1.3, (0.15, 1.2, 40.0, 2e3, 5e7)),
+    (45.0, (0.3, 6.0)),
+    (900.0, (0.4,)),
+    (1.1, (0.3, 2.0, 1e-31)),
+])
+def test_jk_integer_scalars(dist, exps):
+    rng = np.random.default_rng(int(dist * 10) + len(exps))
+    axis = np.array([0.48, -0.6, 0.64])
+    shells = [(a, l, np.array(exps), rng.uniform(0.2, 1.0, len(exps))) for a in (0, 1) for l in (0, 1)]
+    shells += [(0, 2, np.array(exps[:1]), np.ones(1)), (1, 3, np.array(exps[-1:]), np.ones(1))]
+    m = custom_molecule(np.array([[0.1, 0.2, -0.3], axis * dist + [0.1, 0.2, -0.3]]), shells)
+    m.D = random_psd_density(m.nbf, max(2, m.nbf // 3), rng, 1)
+    _check(m)
+
+
+def test_batch_with_a_plan_outside_the_integer_range():
+    rng = np.random.default_rng(3)
+    mols, plans = [], []
+    for top in (4.0, 1e-31):
+        m = custom_molecule(rng.uniform(-1, 1, (2, 3)), [(a, l, np.array([0.4, top]), np.array([0.7, 0.4]))
+                                                         for a in (0, 1) for l in (0, 1)])
+        m.D = random_psd_density(m.nbf, 2, rng, 1)
+        mols.append(m)
+        plans.append(pkg.Plan(m, tau=0.0))
+    Js, Ks = pkg.Batch().jk(plans, [torch.from_numpy(m.D).cuda() for m in mols])
+    for m, J, K in zip(mols, Js, Ks):
+        Jr, Kr, _ = oracle.jk(m, tau=0.0)
+        for got, ref in ((J, Jr), (K, Kr)):
+            assert np.abs(got.cpu().numpy() - ref).max() <= 1e-12 * np.abs(ref).max()
