@@ -1643,7 +1643,7 @@ eri_status eri_jk_grad(eri_plan* p, const double* D, double* gJ, double* gK, voi
   if (!p) return fail(ERI_ERR_ARG, "plan is NULL");
   if (!D || !gJ || !gK) return fail(ERI_ERR_ARG, "D, gJ and gK must be non-NULL");
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  struct GL { int X, Y, ts, grid, smem; long long nt; };
+  struct GL { int X, Y, ts, grid, smem; long long nt; int qsplit; };
   std::vector<GL> ls;
   size_t need = 0, maxnt = 1;
   for (int X = 0; X < ERI_NPAIRTYPE; ++X) {
@@ -1654,7 +1654,7 @@ eri_status eri_jk_grad(eri_plan* p, const double* D, double* gJ, double* gK, voi
       const long long nt = (X == Y) ? nx * (nx + 1) / 2 : nx * ny;
       if ((unsigned long long)nt > 0xffffffffULL) return fail(ERI_ERR_ARG, "class task space above 2^32");
       const GradDesc& g = p->dev->gclasses[X][Y];
-      GL l{X, Y, p->dev->gts[X][Y], 0, 0, nt};
+      GL l{X, Y, p->dev->gts[X][Y], 0, 0, nt, 1};
       const int tpb = 128 / l.ts;
       l.smem = (int)(sizeof(double) * (size_t)g.team_doubles * tpb);
       if (l.smem > 200 * 1024)
@@ -1662,7 +1662,9 @@ eri_status eri_jk_grad(eri_plan* p, const double* D, double* gJ, double* gK, voi
       int bps = 0;
       CUDA_TRY(erik_grad_blocks_per_sm(l.ts, l.smem, &bps));
       if (bps < 1) bps = 1;
-      l.grid = (int)std::max(1LL, std::min((long long)p->dev->sms * bps, (nt + tpb - 1) / tpb));
+      const long long full = (long long)p->dev->sms * bps;
+      l.qsplit = choose_qsplit(nt, full * tpb, p->type_maxprim[X] * p->type_maxprim[Y], g.bp);
+      l.grid = (int)std::max(1LL, std::min(full, (nt * l.qsplit + tpb - 1) / tpb));
       need = std::max(need, (size_t)l.grid * tpb * (size_t)g.scratch_per_team);
       maxnt = std::max(maxnt, (size_t)nt);
       ls.push_back(l);
@@ -1721,12 +1723,15 @@ eri_status eri_jk_grad(eri_plan* p, const double* D, double* gJ, double* gK, voi
     a.counter = p->d_counters + li;
     a.scratch = p->d_scratch + (size_t)sidx * need;
     a.stats = p->d_gstats;
-    unsigned long long* cnt = p->d_tcount + 2 * li;
-    CUDA_TRY(erik_launch_compact(&a, tlist_l, (unsigned long long)l.nt, cnt, tiles_l, 0, sl));
-    a.tlist = tlist_l;
-    a.list_cap = (unsigned long long)l.nt;
-    a.from_back = 0;
-    a.tcount = cnt;
+    a.qsplit = l.qsplit;
+    if (l.nt > kListMinTasks) {
+      unsigned long long* cnt = p->d_tcount + 2 * li;
+      CUDA_TRY(erik_launch_compact(&a, tlist_l, (unsigned long long)l.nt, cnt, tiles_l, 0, sl));
+      a.tlist = tlist_l;
+      a.list_cap = (unsigned long long)l.nt;
+      a.from_back = 0;
+      a.tcount = cnt;
+    }
     GradArgs ga;
     memset(&ga, 0, sizeof(ga));
     ga.k = a;
