@@ -815,6 +815,7 @@ struct eri_plan {
   // kept pairs (Q > tau)
   int type_off[ERI_NPAIRTYPE] = {0}, type_cnt[ERI_NPAIRTYPE] = {0};
   int type_maxprim[ERI_NPAIRTYPE] = {0};   // most primitive pairs of a kept pair, per type
+  long long type_sumprim[ERI_NPAIRTYPE] = {0};   // primitive pairs of the kept pairs, per type
   double type_spread[ERI_NPAIRTYPE] = {0}; // (l0 + l1) / 2 log2 of the largest ratio of a kept pair's zeta
   int npairs_kept = 0;
   std::vector<double> Q;             // [nshell*nshell]
@@ -1087,10 +1088,30 @@ constexpr long long kListMinTasks = 8192;
 // digesting its partial [e0|f0] (the transfer relations and digestion are linear).
 // teams: the teams a full grid holds; minq: the fewest primitive quartets worth a task (a
 // batch of the team kernel).
-int choose_qsplit(long long nt, long long teams, int maxq, int minq) {
-  if (nt <= 0 || maxq <= minq || nt * 2 > teams) return 1;
-  const long long q = (teams + nt - 1) / nt;
-  return (int)std::max(1LL, std::min<long long>({q, (long long)(maxq / std::max(1, minq)), 64LL}));
+// A class with quartets enough to fill the grid is split as well when its deepest quartet (maxq) is
+// over twice the mean load of a team (work / teams primitive quartets): the launch would wait for
+// it.  If a task costs `fixed` primitive quartets beside its own, maxq / q + fixed q nt / teams is
+// least at q = sqrt(maxq teams / (fixed nt)).  fixed was fitted per kernel, since it also stands for
+// the atomics and for the batches a short range leaves part empty.  Unsplit, then by fixed:
+//   one-lane  8:  nine molecules of 5-11 atoms in one batch 13.4 ms; 4, 8, 12, 40 give 10.0, 10.1,
+//                 10.6, 12.4; J alone of 27 atoms 27.3 ms; 2, 4, 8, 12 give 28.8, 27.7, 27.5, 27.3
+//   team     80:  5 atoms, spd, UHF 29.0 ms; 8, 24, 80 give 17.5, 15.6, 14.6
+//   gradient 24:  4 atoms with f and g shells 199 ms; 4, 8, 16, 32 give 228, 191, 172, 182;
+//                 5 atoms 5.28 ms; 4, 8, 16, 32 give 6.07, 5.35, 4.79, 4.61
+// Split where the quartet is over the mean load but not over twice it, J alone of 27 atoms is 2 %
+// slower (one-lane 4: 28.3 against 27.7 ms) and nothing else is faster.
+constexpr double FIXED_LANE = 8.0, FIXED_TEAM = 80.0, FIXED_GRAD = 24.0;
+int choose_qsplit(long long nt, long long teams, int maxq, int minq, double work, double fixed) {
+  if (nt <= 0 || maxq <= minq) return 1;
+  double q = nt * 2 > teams ? 1.0 : (double)((teams + nt - 1) / nt);
+  const double deep = (double)maxq * (double)teams;
+  if (deep > 2.0 * work) q = std::max(q, std::sqrt(deep / (fixed * (double)nt)));
+  return (int)std::max(1.0, std::min({q, (double)(maxq / std::max(1, minq)), 64.0}));
+}
+
+// Primitive quartets of a class's candidate quartets.
+double class_work(const eri_plan* p, int X, int Y) {
+  return (X == Y ? 0.5 : 1.0) * (double)p->type_sumprim[X] * (double)p->type_sumprim[Y];
 }
 
 // Kernel, split, grid and shared memory of a J/K launch over l->nt candidate quartets of at most
@@ -1098,8 +1119,12 @@ int choose_qsplit(long long nt, long long teams, int maxq, int minq) {
 // per quartet (FP32: whenever one exists; FP64: in integers when fx_ok; spread: type_spread of the
 // class's wider type), else for FP64 the fixed-point assembly where the
 // class has one, else the FP64 / FP32 class kernel.
-eri_status shape_launch(eri_plan* p, int maxq, bool fx_ok, double spread, Launch* l) {
+eri_status shape_launch(eri_plan* p, int maxq, double work, bool fx_ok, double spread, Launch* l) {
   const ClassDesc& cd = p->dev->classes[l->X][l->Y];
+  // FP32 launches are split only to fill the grid: their sums over primitive quartets are FP32, and
+  // further ranges moved mixed J / K by 2e-10 to over 1e-9 of the largest element (41 atoms: also
+  // 77.4 instead of 74.6 ms).
+  if (l->fp32) work = HUGE_VAL;
   if ((l->fp32 || p->dev->ts[l->X][l->Y] == 1) && erik_small_available(cd.la, cd.lb, cd.lc, cd.ld, l->fp32)) {
     int bps = 0;
     l->small = !l->fp32 && fx_ok ? 2 : 1;
@@ -1109,7 +1134,7 @@ eri_status shape_launch(eri_plan* p, int maxq, bool fx_ok, double spread, Launch
       CUDA_TRY(erik_small_blocks_per_sm(cd.la, cd.lb, cd.lc, cd.ld, l->fp32, &bps));
     const long long full = (long long)p->dev->sms * std::max(bps, 1);
     l->ts = 1;
-    l->qsplit = choose_qsplit(l->nt, full * 128, maxq, 2);
+    l->qsplit = choose_qsplit(l->nt, full * 128, maxq, 2, work, FIXED_LANE);
     l->grid = (int)std::max(1LL, std::min(full, (l->nt * l->qsplit + 127) / 128));
     l->smem = 0;
     return ERI_OK;
@@ -1119,7 +1144,8 @@ eri_status shape_launch(eri_plan* p, int maxq, bool fx_ok, double spread, Launch
   // a full grid first: the teams it holds decide the split, the split the grid
   eri_status s = launch_shape(p, l->X, l->Y, l->fp32, l->fixed, 1LL << 40, &l->grid, &l->smem, &l->ts);
   if (s != ERI_OK) return s;
-  l->qsplit = choose_qsplit(l->nt, (long long)l->grid * (128 / l->ts), maxq, l->fp32 || !c.xy ? c.bp : c.bp_xy);
+  l->qsplit = choose_qsplit(l->nt, (long long)l->grid * (128 / l->ts), maxq, l->fp32 || !c.xy ? c.bp : c.bp_xy, work,
+                           FIXED_TEAM);
   return launch_shape(p, l->X, l->Y, l->fp32, l->fixed, l->nt * l->qsplit, &l->grid, &l->smem, &l->ts);
 }
 
@@ -1168,7 +1194,7 @@ eri_status plan_launches(eri_plan* p, size_t max_scratch, std::vector<Launch>* o
       const int np = (nprec == 2 && fp32_pays(p, X, Y, nt)) ? 2 : 1;
       for (int fp32 = 0; fp32 < np; ++fp32) {
         Launch l{X, Y, fp32, 0, 0, 0, nt, 0, np == 2 ? 1 : 0, 1, 0};
-        eri_status s = shape_launch(p, p->type_maxprim[X] * p->type_maxprim[Y], p->fx_ok,
+        eri_status s = shape_launch(p, p->type_maxprim[X] * p->type_maxprim[Y], class_work(p, X, Y), p->fx_ok,
                                     std::max(p->type_spread[X], p->type_spread[Y]), &l);
         if (s != ERI_OK) return s;
         if (max_scratch > 0) {
@@ -1601,6 +1627,7 @@ eri_status eri_plan_create(const eri_basis* basis, const eri_opts* opts, void* c
       if (sp.Q > p->opts.screen_thresh) {
         kept.push_back(sp);
         p->type_maxprim[X] = std::max(p->type_maxprim[X], sp.nprim);
+        p->type_sumprim[X] += sp.nprim;
         double zlo = p->prims[sp.prim_off].zeta, zhi = zlo;
         for (int q = 1; q < sp.nprim; ++q) {
           zlo = std::min(zlo, p->prims[sp.prim_off + q].zeta);
@@ -1663,7 +1690,8 @@ eri_status eri_jk_grad(eri_plan* p, const double* D, double* gJ, double* gK, voi
       CUDA_TRY(erik_grad_blocks_per_sm(l.ts, l.smem, &bps));
       if (bps < 1) bps = 1;
       const long long full = (long long)p->dev->sms * bps;
-      l.qsplit = choose_qsplit(nt, full * tpb, p->type_maxprim[X] * p->type_maxprim[Y], g.bp);
+      l.qsplit = choose_qsplit(nt, full * tpb, p->type_maxprim[X] * p->type_maxprim[Y], g.bp,
+                                     class_work(p, X, Y), FIXED_GRAD);
       l.grid = (int)std::max(1LL, std::min(full, (nt * l.qsplit + tpb - 1) / tpb));
       need = std::max(need, (size_t)l.grid * tpb * (size_t)g.scratch_per_team);
       maxnt = std::max(maxnt, (size_t)nt);
@@ -2275,17 +2303,18 @@ eri_status eri_jk_batch(eri_batch* b, int njobs, eri_plan* const* plans, const d
   if ((s = ensure_batch_buf(b, &b->d_jobs, &b->jobs_cap, (size_t)njobs, st)) != ERI_OK) return s;
   CUDA_TRY(cudaMemcpyAsync(b->d_jobs, jobs.data(), sizeof(JobDesc) * njobs, cudaMemcpyHostToDevice, st));
   // ---- classes present in any job, their merged capacities and launch shapes
-  struct BL { int X, Y; long long total; long long maxnt; int any_fp32, maxq; double spread; };
+  struct BL { int X, Y; long long total; long long maxnt; int any_fp32, maxq; double spread, work; };
   std::vector<BL> cls;
   for (int X = 0; X < ERI_NPAIRTYPE; ++X)
     for (int Y = 0; Y <= X; ++Y) {
       long long tot = 0, mx = 0;
       int any32 = 0, maxq = 1;
-      double spread = 0.0;
+      double spread = 0.0, work = 0.0;
       for (int j = 0; j < njobs; ++j) {
         const long long nx = plans[j]->type_cnt[X], ny = plans[j]->type_cnt[Y];
         if (!nx || !ny) continue;
         maxq = std::max(maxq, plans[j]->type_maxprim[X] * plans[j]->type_maxprim[Y]);
+        work += class_work(plans[j], X, Y);
         spread = std::max(spread, std::max(plans[j]->type_spread[X], plans[j]->type_spread[Y]));
         const long long nt = (X == Y) ? nx * (nx + 1) / 2 : nx * ny;
         if ((unsigned long long)nt > 0xffffffffULL) return fail(ERI_ERR_ARG, "job %d has more than 2^32 tasks in a class", j);
@@ -2293,7 +2322,7 @@ eri_status eri_jk_batch(eri_batch* b, int njobs, eri_plan* const* plans, const d
         mx = std::max(mx, nt);
         if (plans[j]->opts.precision == ERI_MIXED && fp32_pays(plans[j], X, Y, nt)) any32 = 1;
       }
-      if (tot) cls.push_back({X, Y, tot, mx, any32, maxq, spread});
+      if (tot) cls.push_back({X, Y, tot, mx, any32, maxq, spread, work});
     }
   size_t cap = 1, tcap = 2, need = 0;
   std::vector<Launch> launches;
@@ -2303,7 +2332,7 @@ eri_status eri_jk_batch(eri_batch* b, int njobs, eri_plan* const* plans, const d
     for (int fp32 = 0; fp32 < (c.any_fp32 ? 2 : 1); ++fp32) {
       // as in eri_jk, over the jobs' merged quartets
       Launch l{c.X, c.Y, fp32, 0, 0, 0, c.total, 0, 0, 1, 0};
-      if ((s = shape_launch(p0, c.maxq, fx_ok, c.spread, &l)) != ERI_OK) return s;
+      if ((s = shape_launch(p0, c.maxq, c.work, fx_ok, c.spread, &l)) != ERI_OK) return s;
       need = std::max(need, (size_t)l.grid * block_scratch(p0, l));
       launches.push_back(l);
     }

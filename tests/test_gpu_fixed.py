@@ -94,3 +94,44 @@ def test_batch_with_a_plan_outside_the_integer_range():
         Jr, Kr, _ = oracle.jk(m, tau=0.0)
         for got, ref in ((J, Jr), (K, Kr)):
             assert np.abs(got.cpu().numpy() - ref).max() <= 1e-12 * np.abs(ref).max()
+
+
+def _uncontracted(coords, shells, D):
+    """The molecule of the shells' primitives, and D (of s and p functions) in its functions."""
+    prims, cols, n = [], [], 0
+    for a, l, e, c in shells:
+        S = (2.0 * np.sqrt(np.outer(e, e)) / np.add.outer(e, e)) ** (l + 1.5)
+        w = c / np.sqrt(c @ S @ c)
+        for comp in range(2 * l + 1):
+            cols.append({n + k * (2 * l + 1) + comp: w[k] for k in range(len(e))})
+        prims += [(a, l, e[k:k + 1], np.ones(1)) for k in range(len(e))]
+        n += len(e) * (2 * l + 1)
+    C = np.zeros((n, len(cols)))
+    for j, col in enumerate(cols):
+        for i, v in col.items():
+            C[i, j] = v
+    return custom_molecule(coords, prims), np.ascontiguousarray(C @ D @ C.T)
+
+
+# Classes with quartets enough to fill the grid, a few of them deep (6^4 primitive quartets among
+# quartets of one): the deep ones are split over primitive ranges, the shallow ones have ranges
+# without a primitive.  ns s1 shells and np_ p1 shells around one s6 and one p6 shell; the
+# tolerance as above, of the gradient as in its own tests.
+@pytest.mark.parametrize("ns,np_", [(24, 13), (30, 2)])
+def test_deep_quartets_in_a_full_grid(ns, np_):
+    rng = np.random.default_rng(ns)
+    coords = rng.uniform(-2, 2, (6, 3))
+    one = lambda l, a: (a, l, rng.uniform(0.2, 2.0, 1), np.ones(1))  # noqa: E731
+    shells = [one(0, i % 6) for i in range(ns)] + [one(1, i % 6) for i in range(np_)]
+    deep = 0.15 * 4.0 ** np.arange(6)
+    shells += [(1, 0, deep, rng.uniform(0.1, 0.6, 6)), (4, 1, deep, rng.uniform(0.1, 0.6, 6))]
+    shells.sort(key=lambda s: s[0])
+    m = custom_molecule(coords, shells)
+    m.D = random_psd_density(m.nbf, 5, rng, 1)
+    _check(m)
+    # the gradient against that of the same density in the primitives as shells of their own, where
+    # no quartet is deep
+    got = pkg.Plan(m, tau=0.0).jk_grad(torch.from_numpy(m.D[0]).cuda())
+    u, D = _uncontracted(coords, shells, m.D[0])
+    for g, r in zip(got, pkg.Plan(u, tau=0.0).jk_grad(torch.from_numpy(D).cuda())):
+        assert (g - r).abs().max() <= 1e-10 * max(1.0, float(r.abs().max()))
