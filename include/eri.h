@@ -230,7 +230,7 @@ eri_status eri_rys_roots(int N, int n, const double* T, double* u, double* w);
 /* Per-launch record of the last eri_jk call when profiling is on. */
 typedef struct {
   int la, lb, lc, ld;             /* class of the launch */
-  int team_size;                  /* threads per shell quartet (1, 2, 4, 8, 32 or 128) */
+  int team_size;                  /* threads per shell quartet (1, 2, 4, 8, 16, 32 or 128) */
   int grid;                       /* blocks launched */
   float ms;                       /* CUDA-event time of the launch on the call's stream */
   long long quartets;             /* shell quartets evaluated (after screening) */
@@ -238,14 +238,16 @@ typedef struct {
   double model_flops;             /* arithmetic of the launch by the kernel's operation count (FP64 + FP32) */
   double model_flops_fp32;        /* its FP32 part */
   int fp32;                       /* 1 for the FP32 path of ERI_MIXED */
-  int specialised;                /* 1 for a compile-time specialised small-class kernel */
+  int specialised;                /* 1 for a compile-time specialised small-class kernel (FP64
+                                     launches in integer arithmetic where the exponents allow) */
   int shared_products;            /* 1 when the launch formed each I_x I_y product once per team in
                                      shared memory; 0 for lane programs (products reused within a
                                      lane) */
   int compiled_class;             /* 1 when the team kernel was compiled for this one class (its root
                                      count and recurrence sizes constants) */
   int quartet_split;              /* tasks per shell quartet: > 1 when the class had too few quartets
-                                     to fill the GPU and each ran as that many ranges of its
+                                     to fill the GPU, or some far deeper than a
+                                     team's mean load, and each ran as that many ranges of its
                                      primitive quartets, each digesting its partial sums */
   int listed;                     /* 1 when the kept quartets were compacted into a task list before
                                      the launch; 0 when the kernel screened the class's candidates */

@@ -21,7 +21,8 @@
 //      on the bra and the same with C-D on the ket turn [e0|f0] into (ab|cd);
 //   3. digestion into J~ and K~ with the six updates of Alg. 2 and the
 //      permutation weights of the unique quartet, by FP64 atomicAdd.
-// The Rys roots, weights and recurrences are FP64 throughout.
+// Roots and weights are FP64 values of 64-bit fixed-point sums (rys_fixed.h), the recurrences FP64.
+// FP64 J/K launches of classes up to L = 8 run eri_fixed.cu or eri_small.cu instead.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
