@@ -730,7 +730,7 @@ eri_status device_init(int dev, DeviceState** out) {
 
 // Operation count of the class kernel's algorithm (an FMA counts as 2), mirroring
 // eri_kernels.cu, split by pipe: per primitive quartet the Gaussian-product scalars and T,
-// per root the two degree-11 Horner sums (FP64 always) and the recurrence coefficients,
+// per root the two Horner sums (in FP64 or 64-bit integers) and the recurrence coefficients,
 // the three 2D tables and the Eq. 1 products (a multiply and an FMA per [e0|f0] value and
 // root); per contracted quartet the transfer relations and the six digestion updates (both
 // FP64 always).  fp32 = 1 counts the FP32 path of the mixed mode.
@@ -1483,6 +1483,8 @@ eri_status eri_plan_create(const eri_basis* basis, const eri_opts* opts, void* c
         }
       if (t.keep.empty()) t.keep.push_back(best);
       // by total exponent: the fixed-point kernels scale batches of neighbours together
+      // mixed plans keep the shells' order: the FP32 launches add their FP32 sums in it
+      if (p->opts.precision != ERI_MIXED)
       std::stable_sort(t.keep.begin(), t.keep.end(), [&](int c0, int c1) {
         const int nb = p->sh_nprim[b];
         const double z0 = p->exps[p->sh_off[a] + c0 / nb] + p->exps[p->sh_off[b] + c0 % nb];
@@ -1633,7 +1635,9 @@ eri_status eri_plan_create(const eri_basis* basis, const eri_opts* opts, void* c
           zlo = std::min(zlo, p->prims[sp.prim_off + q].zeta);
           zhi = std::max(zhi, p->prims[sp.prim_off + q].zeta);
         }
-        p->type_spread[X] = std::max(p->type_spread[X], 0.5 * (p->sh_l[sp.sh0] + p->sh_l[sp.sh1]) * std::log2(zhi / zlo));
+        // unsorted, a batch of a mixed plan holds exponents further apart: 6 binades less allowed
+        const double spread = 0.5 * (p->sh_l[sp.sh0] + p->sh_l[sp.sh1]) * std::log2(zhi / zlo);
+        p->type_spread[X] = std::max(p->type_spread[X], spread + (p->opts.precision == ERI_MIXED ? 6.0 : 0.0));
       }
     }
     p->type_cnt[X] = (int)kept.size() - p->type_off[X];
