@@ -526,7 +526,9 @@ __global__ void __launch_bounds__(TPB, (SmallFx<LA, LB, LC, LD>::blocks)) eri_sm
           int64_t um, wm;
           int ue, we;
           sx_root(a.rys_coef, reinterpret_cast<const longlong2*>(a.rys_asym), N, s, n, um, ue, wm, we);
-          const int64_t w60 = sx_shift(wm, 2 - we);
+          // in units of 2^rTe, about 1/sqrt(T), in the large-T limit: the weight keeps its 60 bits there
+          // (as an absolute 2^-60 it lost log2(T) / 2 of them, 2.3e-13 of a repulsion at T = 1e11)
+          const int64_t w60 = sx_shift(wm, 2 - (we - s.rTe));
           int64_t C6[3] = {0, 0, 0}, Cp6[3] = {0, 0, 0}, b10 = 0, b01 = 0, b00 = 0;
           if (LE > 0) {
             const int64_t fm = sx_mulm(um, rzm);
@@ -614,7 +616,7 @@ __global__ void __launch_bounds__(TPB, (SmallFx<LA, LB, LC, LD>::blocks)) eri_sm
         for (int i = 0; i <= LB; ++i)
 #pragma unroll
           for (int j = 0; j <= LD; ++j)
-            sc[i * (LD + 1) + j] = scale_pow2(theta, (x.a - sa) * (LA + i) + (y.a - sb) * (LC + j) - 60 + wl);
+            sc[i * (LD + 1) + j] = scale_pow2(theta, (x.a - sa) * (LA + i) + (y.a - sb) * (LC + j) + s.rTe - 60 + wl);
         sfor<0, NOUT>([&](auto oc) {
           constexpr int o = decltype(oc)::value;
           const double d = __ll2double_rn(acc[o]);
