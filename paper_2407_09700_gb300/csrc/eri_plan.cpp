@@ -817,6 +817,8 @@ struct eri_plan {
   int type_maxprim[ERI_NPAIRTYPE] = {0};   // most primitive pairs of a kept pair, per type
   long long type_sumprim[ERI_NPAIRTYPE] = {0};   // primitive pairs of the kept pairs, per type
   double type_spread[ERI_NPAIRTYPE] = {0}; // (l0 + l1) / 2 log2 of the largest ratio of a kept pair's zeta
+  double type_rt[ERI_NPAIRTYPE] = {0};     // l0 + l1 > 0: bound of zeta |P - Q|^2 over the kept pairs' primitives
+  double diag2 = 0.0;                // squared diagonal of the atoms' bounding box
   int npairs_kept = 0;
   std::vector<double> Q;             // [nshell*nshell]
   std::vector<double> Qe;            // [nshell*nshell] transfer-aware factors of the mixed split
@@ -1021,6 +1023,7 @@ void make_prim_fx(eri_plan* p, PrimFx* out) {
     }
     mid[x] = std::nearbyint(0.5 * (lo[x] + hi[x]));
     ext = std::max(ext, std::max(hi[x] - mid[x], mid[x] - lo[x]));
+    p->diag2 += (hi[x] - lo[x]) * (hi[x] - lo[x]);
   }
   int e = 0;
   (void)std::frexp(2.0 * ext, &e);                       // |P - Q| <= 2 ext < 2^e
@@ -1114,12 +1117,17 @@ double class_work(const eri_plan* p, int X, int Y) {
   return (X == Y ? 0.5 : 1.0) * (double)p->type_sumprim[X] * (double)p->type_sumprim[Y];
 }
 
+// Whether a one-lane FP64 launch of class (X|Y) holds FP64's accuracy in integers (eri_scalar.cuh).
+bool fx_class(const eri_plan* p, int X, int Y) {
+  return p->fx_ok && std::max(p->type_rt[X], p->type_rt[Y]) <= SX_TMAX;
+}
+
 // Kernel, split, grid and shared memory of a J/K launch over l->nt candidate quartets of at most
 // maxq primitive quartets: the specialised one-lane kernel where the class runs with one lane
-// per quartet (FP32: whenever one exists; FP64: in integers when fx_ok; spread: type_spread of the
+// per quartet (FP32: whenever one exists; FP64: in integers when fx, see fx_class; spread: type_spread of the
 // class's wider type), else for FP64 the fixed-point assembly where the
 // class has one, else the FP64 / FP32 class kernel.
-eri_status shape_launch(eri_plan* p, int maxq, double work, bool fx_ok, double spread, Launch* l) {
+eri_status shape_launch(eri_plan* p, int maxq, double work, bool fx, double spread, Launch* l) {
   const ClassDesc& cd = p->dev->classes[l->X][l->Y];
   // FP32 launches are split only to fill the grid: their sums over primitive quartets are FP32, and
   // further ranges moved mixed J / K by 2e-10 to over 1e-9 of the largest element (41 atoms: also
@@ -1127,7 +1135,7 @@ eri_status shape_launch(eri_plan* p, int maxq, double work, bool fx_ok, double s
   if (l->fp32) work = HUGE_VAL;
   if ((l->fp32 || p->dev->ts[l->X][l->Y] == 1) && erik_small_available(cd.la, cd.lb, cd.lc, cd.ld, l->fp32)) {
     int bps = 0;
-    l->small = !l->fp32 && fx_ok ? 2 : 1;
+    l->small = !l->fp32 && fx ? 2 : 1;
     if (l->small == 2)
       CUDA_TRY(erik_small_fx_blocks_per_sm(cd.la, cd.lb, cd.lc, cd.ld, &bps));
     else
@@ -1194,7 +1202,7 @@ eri_status plan_launches(eri_plan* p, size_t max_scratch, std::vector<Launch>* o
       const int np = (nprec == 2 && fp32_pays(p, X, Y, nt)) ? 2 : 1;
       for (int fp32 = 0; fp32 < np; ++fp32) {
         Launch l{X, Y, fp32, 0, 0, 0, nt, 0, np == 2 ? 1 : 0, 1, 0};
-        eri_status s = shape_launch(p, p->type_maxprim[X] * p->type_maxprim[Y], class_work(p, X, Y), p->fx_ok,
+        eri_status s = shape_launch(p, p->type_maxprim[X] * p->type_maxprim[Y], class_work(p, X, Y), fx_class(p, X, Y),
                                     std::max(p->type_spread[X], p->type_spread[Y]), &l);
         if (s != ERI_OK) return s;
         if (max_scratch > 0) {
@@ -1638,6 +1646,7 @@ eri_status eri_plan_create(const eri_basis* basis, const eri_opts* opts, void* c
         // unsorted, a batch of a mixed plan holds exponents further apart: 6 binades less allowed
         const double spread = 0.5 * (p->sh_l[sp.sh0] + p->sh_l[sp.sh1]) * std::log2(zhi / zlo);
         p->type_spread[X] = std::max(p->type_spread[X], spread + (p->opts.precision == ERI_MIXED ? 6.0 : 0.0));
+        if (p->sh_l[sp.sh0] > 0) p->type_rt[X] = std::max(p->type_rt[X], zhi * p->diag2);
       }
     }
     p->type_cnt[X] = (int)kept.size() - p->type_off[X];
@@ -2273,10 +2282,8 @@ eri_status eri_jk_batch(eri_batch* b, int njobs, eri_plan* const* plans, const d
   eri_plan* p0 = plans[0];
   // ---- job descriptors
   std::vector<JobDesc> jobs(njobs);
-  bool fx_ok = true;
   for (int j = 0; j < njobs; ++j) {
     eri_plan* p = plans[j];
-    fx_ok = fx_ok && p->fx_ok;
     JobDesc& jd = jobs[j];
     memset(&jd, 0, sizeof(jd));
     jd.pairs = p->d_pairs;
@@ -2307,18 +2314,20 @@ eri_status eri_jk_batch(eri_batch* b, int njobs, eri_plan* const* plans, const d
   if ((s = ensure_batch_buf(b, &b->d_jobs, &b->jobs_cap, (size_t)njobs, st)) != ERI_OK) return s;
   CUDA_TRY(cudaMemcpyAsync(b->d_jobs, jobs.data(), sizeof(JobDesc) * njobs, cudaMemcpyHostToDevice, st));
   // ---- classes present in any job, their merged capacities and launch shapes
-  struct BL { int X, Y; long long total; long long maxnt; int any_fp32, maxq; double spread, work; };
+  struct BL { int X, Y; long long total; long long maxnt; int any_fp32, maxq; double spread, work; bool fx; };
   std::vector<BL> cls;
   for (int X = 0; X < ERI_NPAIRTYPE; ++X)
     for (int Y = 0; Y <= X; ++Y) {
       long long tot = 0, mx = 0;
       int any32 = 0, maxq = 1;
       double spread = 0.0, work = 0.0;
+      bool fx = true;
       for (int j = 0; j < njobs; ++j) {
         const long long nx = plans[j]->type_cnt[X], ny = plans[j]->type_cnt[Y];
         if (!nx || !ny) continue;
         maxq = std::max(maxq, plans[j]->type_maxprim[X] * plans[j]->type_maxprim[Y]);
         work += class_work(plans[j], X, Y);
+        fx = fx && fx_class(plans[j], X, Y);
         spread = std::max(spread, std::max(plans[j]->type_spread[X], plans[j]->type_spread[Y]));
         const long long nt = (X == Y) ? nx * (nx + 1) / 2 : nx * ny;
         if ((unsigned long long)nt > 0xffffffffULL) return fail(ERI_ERR_ARG, "job %d has more than 2^32 tasks in a class", j);
@@ -2326,7 +2335,7 @@ eri_status eri_jk_batch(eri_batch* b, int njobs, eri_plan* const* plans, const d
         mx = std::max(mx, nt);
         if (plans[j]->opts.precision == ERI_MIXED && fp32_pays(plans[j], X, Y, nt)) any32 = 1;
       }
-      if (tot) cls.push_back({X, Y, tot, mx, any32, maxq, spread, work});
+      if (tot) cls.push_back({X, Y, tot, mx, any32, maxq, spread, work, fx});
     }
   size_t cap = 1, tcap = 2, need = 0;
   std::vector<Launch> launches;
@@ -2336,7 +2345,7 @@ eri_status eri_jk_batch(eri_batch* b, int njobs, eri_plan* const* plans, const d
     for (int fp32 = 0; fp32 < (c.any_fp32 ? 2 : 1); ++fp32) {
       // as in eri_jk, over the jobs' merged quartets
       Launch l{c.X, c.Y, fp32, 0, 0, 0, c.total, 0, 0, 1, 0};
-      if ((s = shape_launch(p0, c.maxq, c.work, fx_ok, c.spread, &l)) != ERI_OK) return s;
+      if ((s = shape_launch(p0, c.maxq, c.work, c.fx, c.spread, &l)) != ERI_OK) return s;
       need = std::max(need, (size_t)l.grid * block_scratch(p0, l));
       launches.push_back(l);
     }

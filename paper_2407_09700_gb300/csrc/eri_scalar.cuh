@@ -21,6 +21,12 @@
 #include "eri_internal.h"
 #include "rys_fixed.h"
 
+// Largest zeta |P - Q|^2 of the FP64 launches with p or higher functions.  C of a tight pair on one
+// centre is about 1 / (zeta |P - Q|), sqrt(T) below its unit of length, so that a (ps|ss) carries
+// about 2^-57.6 sqrt(zeta |P - Q|^2): 1.7e-15 at this limit (5.3e-14 measured at 1.3e8, 4.4e-13 at 1.3e10),
+// where FP64 keeps 1e-15.  Wider classes run in FP64.
+#define SX_TMAX 131072.0
+
 #define SX_M30 0x3fffffff
 #define SX_M31 0x7fffffff
 

@@ -44,3 +44,12 @@ def test_repulsion_of_tight_shells(zeta):
     got, want = _separated(zeta)
     assert abs(got[0] / want[0] - 1) <= 4e-15
     assert abs(got[2] / want[2] - 1) <= 4e-15
+
+
+# (ps|ss), a dipole's repulsion, is about 1 / sqrt(zeta R^2) of the unit its C is held in; a few units of
+# 2^-60 leave 2^-57.6 sqrt(zeta R^2), 1.7e-15 at the largest zeta R^2 that the integers take (2^17, between
+# 1e3 and 2e3 here), beside the roundings of the other elements: twice the sum of both.
+@pytest.mark.parametrize("zeta", [1e2, 1e3, 2e3, 1e4, 1e6, 1e8, 1e12])
+def test_dipole_of_tight_shells(zeta):
+    got, want = _separated(zeta)
+    assert abs(got[1] / want[1] - 1) <= 8e-15
