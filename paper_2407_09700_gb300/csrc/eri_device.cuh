@@ -581,7 +581,7 @@ struct TaskCtx {
   const double* D;
   double* J;
   double* K;
-  int nbf, nD, want, pu;
+  int nbf, nD, want, pu, fx64;
 };
 
 __device__ __forceinline__ TaskCtx single_ctx(const KernelArgs& a) {
@@ -591,6 +591,7 @@ __device__ __forceinline__ TaskCtx single_ctx(const KernelArgs& a) {
   c.primsf = a.primsf;
   c.prfx = a.prfx;
   c.pu = a.pu;
+  c.fx64 = a.fx64;
   c.D = a.D;
   c.J = a.J;
   c.K = a.K;
@@ -602,10 +603,10 @@ __device__ __forceinline__ TaskCtx single_ctx(const KernelArgs& a) {
 
 // P - Q of primitive pairs x and y (indices ix, iy): from the integer positions, whose difference is
 // exact (rounding P itself costs 2^-53 |P| bohr, which tight shells see as sqrt(zeta) times that), or
-// from the doubles when the plan has none (pu < 0).
+// from the doubles when the plan's unit is too coarse.
 __device__ __forceinline__ void pair_distance(const TaskCtx& tc, const PrimPair* x, const PrimPair* y, int ix, int iy,
                                               double& d0, double& d1, double& d2) {
-  if (tc.pu >= 0) {
+  if (tc.fx64) {
     const longlong2* p = reinterpret_cast<const longlong2*>(tc.prfx + ix);
     const longlong2* q = reinterpret_cast<const longlong2*>(tc.prfx + iy);
     const longlong2 p0 = __ldg(p), q0 = __ldg(q);
@@ -633,6 +634,7 @@ __device__ __forceinline__ void resolve_task(const KernelArgs& a, long long task
     ctx.primsf = jd.primsf;
     ctx.prfx = jd.prfx;
     ctx.pu = jd.pu;
+    ctx.fx64 = jd.fx64;
     ctx.D = jd.D;
     ctx.J = jd.J;
     ctx.K = jd.K;

@@ -123,7 +123,7 @@ struct JobDesc {
   double* J;
   double* K;
   const struct PrimFx* prfx;
-  int nbf, nD, want, pu;
+  int nbf, nD, want, pu, fx64, pad;
   int type_off[ERI_NPAIRTYPE];
   int type_cnt[ERI_NPAIRTYPE];
 };
@@ -134,7 +134,8 @@ struct KernelArgs {
   const PrimPair* prims;
   const PrimPairF* primsf;     // FP32 shadow (FP32 kernels)
   const PrimFx* prfx;          // integer scalars of the one-lane kernels
-  int pu;                      // unit 2^-pu of PrimFx::P; < 0: the plan has no integer scalars
+  int pu;                      // unit 2^-pu of PrimFx::P
+  int fx64;                    // 1: fine enough for FP64 launches
   // task space: bra pairs [bra0, bra0+nbra), ket pairs [ket0, ket0+nket); tri = same range, ket <= bra
   int bra0, nbra, ket0, nket, tri;
   long long ntask;

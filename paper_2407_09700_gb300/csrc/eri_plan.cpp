@@ -828,8 +828,9 @@ struct eri_plan {
   PrimPair* d_prims = nullptr;
   PrimPairF* d_primsf = nullptr;
   PrimFx* d_prfx = nullptr;
-  int pu = -1;                       // unit 2^-pu of PrimFx::P (< 0: no integer positions)
-  bool fx_ok = true;                 // every exponent within the integer scalars' range
+  int pu = 0;                        // unit 2^-pu of PrimFx::P
+  bool fx_ok = true;                 // the FP32 launches may take the integer scalars
+  bool fx64 = true;                  // the FP64 launches too: positions in units of 2^-SX_PU or finer
   int* d_sh_bf0 = nullptr;
   int* d_sh_n = nullptr;
   int* d_sh_atom = nullptr;
@@ -950,6 +951,7 @@ KernelArgs base_args(eri_plan* p, int X, int Y) {
   a.rys_asym = p->dev->rys_asym + 4 * RYS_ASYM_OFFSET[N];
   a.prfx = p->d_prfx;
   a.pu = p->pu;
+  a.fx64 = p->fx64;
   a.err = p->d_err;
   return a;
 }
@@ -1012,7 +1014,10 @@ eri_status validate_basis(const eri_basis* b) {
 
 
 // Integer shadows of the primitive pairs (eri_scalar.cuh): positions from a point near the
-// molecule's middle in units of 2^-pu that hold every P - Q in 60 bits.
+// molecule's middle in units of 2^-pu that hold every P - Q in 60 bits.  One atom far away makes the
+// unit coarse for all: from SX_PU places on the FP64 launches take it, and the FP32 launches, which
+// round P - Q to 2^-24, from SX_PU32 on.  The exponents' range and the unit's lower end keep every
+// FP32 value made from them normal: T below 2^119, P - Q in units of 2^-99.
 void make_prim_fx(eri_plan* p, PrimFx* out) {
   double lo[3], hi[3], mid[3], ext = 0.0;
   for (int x = 0; x < 3; ++x) {
@@ -1026,9 +1031,10 @@ void make_prim_fx(eri_plan* p, PrimFx* out) {
     p->diag2 += (hi[x] - lo[x]) * (hi[x] - lo[x]);
   }
   int e = 0;
-  (void)std::frexp(2.0 * ext, &e);                       // |P - Q| <= 2 ext < 2^e
+  if (ext > 0x1p-41) (void)std::frexp(std::min(2.0 * ext, 0x1p60), &e);   // |P - Q| <= 2 ext < 2^e
+  else e = -40;
   p->pu = 59 - e;
-  p->fx_ok = e < 59;
+  p->fx_ok = p->pu >= SX_PU32;
   const double upu = p->fx_ok ? sx_pow2(p->pu) : 0.0;
   std::vector<int64_t> org(3 * p->natm, 0);
   if (p->fx_ok)
@@ -1038,7 +1044,7 @@ void make_prim_fx(eri_plan* p, PrimFx* out) {
       const PrimPair& q = p->prims[k];
       PrimFx& f = out[k];
       memset(&f, 0, sizeof(f));
-      if (!(q.zeta > 1e-30 && q.zeta < 1e30) || !std::isfinite(q.E)) {
+      if (!(q.zeta > 1e-18 && q.zeta < 1e18) || !std::isfinite(q.E)) {
         p->fx_ok = false;
         continue;
       }
@@ -1119,7 +1125,7 @@ double class_work(const eri_plan* p, int X, int Y) {
 
 // Whether a one-lane FP64 launch of class (X|Y) holds FP64's accuracy in integers (eri_scalar.cuh).
 bool fx_class(const eri_plan* p, int X, int Y) {
-  return p->fx_ok && std::max(p->type_rt[X], p->type_rt[Y]) <= SX_TMAX;
+  return p->fx64 && std::max(p->type_rt[X], p->type_rt[Y]) <= SX_TMAX;
 }
 
 // Kernel, split, grid and shared memory of a J/K launch over l->nt candidate quartets of at most
@@ -1588,7 +1594,7 @@ eri_status eri_plan_create(const eri_basis* basis, const eri_opts* opts, void* c
   PLAN_TRY(cudaMemcpyAsync(p->d_primsf, primsf.data(), sizeof(PrimPairF) * primsf.size(), cudaMemcpyHostToDevice, st));
   std::vector<PrimFx> prfx(p->prims.size());
   make_prim_fx(p, prfx.data());
-  if (!p->fx_ok) p->pu = -1;
+  p->fx64 = p->fx_ok && p->pu >= SX_PU;
   PLAN_TRY(cudaMemcpyAsync(p->d_prfx, prfx.data(), sizeof(PrimFx) * prfx.size(), cudaMemcpyHostToDevice, st));
   PLAN_TRY(cudaMemcpyAsync(p->d_sh_bf0, p->sh_bf0.data(), sizeof(int) * p->nshell, cudaMemcpyHostToDevice, st));
   PLAN_TRY(cudaMemcpyAsync(p->d_sh_n, sh_n.data(), sizeof(int) * p->nshell, cudaMemcpyHostToDevice, st));
@@ -2291,6 +2297,7 @@ eri_status eri_jk_batch(eri_batch* b, int njobs, eri_plan* const* plans, const d
     jd.primsf = p->d_primsf;
     jd.prfx = p->d_prfx;
     jd.pu = p->pu;
+    jd.fx64 = p->fx64;
     jd.D = D[j];
     jd.J = J[j];
     jd.K = K[j];

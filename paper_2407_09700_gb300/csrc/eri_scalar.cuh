@@ -27,6 +27,12 @@
 // where FP64 keeps 1e-15.  Wider classes run in FP64.
 #define SX_TMAX 131072.0
 
+// Fewest binary places of the positions in FP64 and in FP32 launches (64 and 2^28 bohr to either side of
+// the molecule's middle).  P - Q is off by up to a unit, the coordinates in FP64 by 2^-53 of themselves:
+// with an atom 1e3, 1e5 and 1e7 bohr away the unit cost J of a compact molecule 4e-15, 8e-13 and 6e-11.
+#define SX_PU 52
+#define SX_PU32 30
+
 #define SX_M30 0x3fffffff
 #define SX_M31 0x7fffffff
 

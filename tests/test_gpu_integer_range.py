@@ -53,3 +53,57 @@ def test_repulsion_of_tight_shells(zeta):
 def test_dipole_of_tight_shells(zeta):
     got, want = _separated(zeta)
     assert abs(got[1] / want[1] - 1) <= 8e-15
+
+
+def _cluster(far, rng):
+    """Three atoms with s, p and d shells near the origin and an s function at (far, 0, 0); the
+    cluster's blocks of J and K and its gradients, of a density of its own."""
+    coords = np.vstack([rng.uniform(-1.5, 1.5, (3, 3)), [[far, 0.0, 0.0]]])
+    e = np.array([0.3, 1.9, 11.0])
+    m = custom_molecule(coords, [(a, l, e, np.ones(3)) for a in range(3) for l in (0, 1, 2)] + [(3, 0, e[:1], e[:1])])
+    C = rng.standard_normal((m.nbf - 1, 4)) / 5
+    D = np.zeros((m.nbf, m.nbf))
+    D[:-1, :-1] = C @ C.T
+    D = torch.from_numpy(D).cuda()
+    plan = pkg.Plan(m, tau=0.0)
+    J, K = plan.jk(D)
+    return [x.cpu().numpy()[:-1, :-1] for x in (J, K)] + [g.cpu().numpy()[:3] for g in plan.jk_grad(D)]
+
+
+# A far atom leaves the cluster's values as they are; the bound is that of the sums' own roundings
+# (about 1e4 atomic additions: sqrt(1e4) 2^-53 = 1.1e-14 of the largest element, 2e-15 in practice;
+# gradients cancel to a quarter of their parts).
+@pytest.mark.parametrize("far", [60.0, 300.0, 1e3, 1e5, 1e9, 1e15])
+def test_cluster_with_an_atom_far_away(far):
+    for got, ref, tol in zip(_cluster(far, np.random.default_rng(3)), _cluster(30.0, np.random.default_rng(3)),
+                             (1.1e-14, 1.1e-14, 4.4e-14, 4.4e-14)):
+        assert np.abs(got - ref).max() <= tol * np.abs(ref).max()
+
+
+# FP32 launches (a threshold that takes every quartet): T = 1e40, where u would leave FP32's range, positions in
+# coarse units, and the large-T limit; each block of the first atom in the field of the second's s
+# function by its own size, FP32 sums to 1e-5.
+@pytest.mark.parametrize("zeta,R", [(1e22, 1e9), (3.0, 1e7), (1e10, 8.0)])
+def test_mixed_at_the_ends_of_fp32(zeta, R):
+    got, ref = _mixed_and_fp64(zeta, R, R)
+    s0, p0 = slice(0, 1), slice(1, 4)
+    for rows, cols in ((s0, s0), (s0, p0), (p0, p0)):
+        g, r = got[rows, cols], ref[rows, cols]
+        assert (g - r).abs().max() <= 1e-5 * r.abs().max()
+
+
+# Centres 1e-30 bohr apart, where the positions' unit would leave it: as for one centre.
+def test_mixed_of_nearly_coincident_centres():
+    got, ref = _mixed_and_fp64(1.0, 1e-30, 0.0)
+    assert (got - ref).abs().max() <= 1e-5 * ref.abs().max()
+
+
+def _mixed_and_fp64(zeta, R, R64):
+    one, J = np.ones(1), []
+    for r, opts in ((R, dict(precision=pkg.ERI_MIXED, mixed_thresh=1e300, mixed_min_tasks=0)), (R64, {})):
+        m = custom_molecule(np.array([[0.0, 0, 0], [r, 0, 0]]),
+                            [(a, l, np.array([zeta]), one) for a in (0, 1) for l in (0, 1)])
+        D = np.zeros((m.nbf, m.nbf))
+        D[-4, -4] = 1.0                           # the second atom's s function
+        J.append(pkg.Plan(m, tau=0.0, **opts).jk(torch.from_numpy(D).cuda())[0])
+    return J
