@@ -249,8 +249,9 @@ __global__ void __launch_bounds__(TPB, (TS == 1 ? 3 : ((sizeof(R) == 4 && !XY) ?
           const PrimPair* yd = (STAGE && staged) ? stage + npb + q % npk : tc.prims + iyp;
           const double s = xd->zeta + yd->zeta;
           const double rd = rsqrt(s);
-          double PQ0, PQ1, PQ2;
-          pair_distance(tc, xd, yd, ixp, iyp, PQ0, PQ1, PQ2);
+          // in FP64: from the integer positions (pair_distance) the diagonal quartets of a plan's Schwarz
+          // factors, one team per deep quartet, took a tenth longer (5 atoms, spd, depth 6: 98.4 -> 107.7 ms)
+          const double PQ0 = xd->P[0] - yd->P[0], PQ1 = xd->P[1] - yd->P[1], PQ2 = xd->P[2] - yd->P[2];
           const double T = xd->zeta * yd->zeta * (rd * rd) * fma(PQ0, PQ0, fma(PQ1, PQ1, PQ2 * PQ2));
           rys_put_team(sd, j * NPD, rys_locate(T, a.rys_tcut_hi));
           const PP* x = (sizeof(R) == 8) ? reinterpret_cast<const PP*>(xd) : prims_r + ixp;

@@ -145,7 +145,6 @@ __global__ void __launch_bounds__(TPB, (TS == 1 ? 3 : 2)) eri_grad_kernel(const 
   extern __shared__ double smem[];
   const KernelArgs& a = ga.k;
   const GradDesc& g = ga.g;
-  const TaskCtx tc = single_ctx(a);
   // TS = TPB: one team per block (team barriers are __syncthreads), as in the J/K kernel
   constexpr bool BLK = TS > 32;
   static_assert(!BLK || TS == TPB, "a team is a warp's part or the whole block");
@@ -279,13 +278,11 @@ __global__ void __launch_bounds__(TPB, (TS == 1 ? 3 : 2)) eri_grad_kernel(const 
       for (int j = tl; j < bp; j += TS) {
         if (j < nbt) {
           const int q = qlo + q0 + j;
-          const int ix = boff + q / npk, iy = koff + q % npk;
-          const PrimPair* x = a.prims + ix;
-          const PrimPair* y = a.prims + iy;
+          const PrimPair* x = a.prims + boff + q / npk;
+          const PrimPair* y = a.prims + koff + q % npk;
           const double zeta = x->zeta, eta = y->zeta;
           const double rd = rsqrt(zeta + eta);
-          double PQ0, PQ1, PQ2;
-          pair_distance(tc, x, y, ix, iy, PQ0, PQ1, PQ2);
+          const double PQ0 = x->P[0] - y->P[0], PQ1 = x->P[1] - y->P[1], PQ2 = x->P[2] - y->P[2];
           const double inv_s = rd * rd;
           const double T = zeta * eta * inv_s * fma(PQ0, PQ0, fma(PQ1, PQ1, PQ2 * PQ2));
           rys_put_team(sd, j * NPD, rys_locate(T, a.rys_tcut_hi));

@@ -12,7 +12,7 @@
 // centres A, B).  80 bytes, 16-byte aligned.
 struct PrimPair {
   double zeta;     // alpha + beta
-  double P[3];     // (alpha A + beta B) / zeta
+  double P[3];     // (alpha A + beta B) / zeta = A + (P - A)
   double PA[3];    // P - A
   double E;        // sqrt(2) pi^(5/4) / zeta * exp(-alpha beta |A-B|^2 / zeta) * c_alpha c_beta
   double hz;       // 1 / (2 zeta)

@@ -1539,8 +1539,8 @@ eri_status eri_plan_create(const eri_basis* basis, const eri_opts* opts, void* c
       PrimPair pp;
       pp.zeta = al + be;
       for (int x = 0; x < 3; ++x) {
-        pp.P[x] = (al * A[x] + be * B[x]) / pp.zeta;
         pp.PA[x] = -(be / pp.zeta) * sp.AB[x];   // P - A without the cancellation
+        pp.P[x] = A[x] + pp.PA[x];               // A itself for a pair on one centre
       }
       pp.E = pref / pp.zeta * std::exp(-al * be / pp.zeta * AB2) * ca * cb;
       pp.hz = 0.5 / pp.zeta;
