@@ -248,6 +248,9 @@ int erik_launch_compact_batched(const struct KernelArgs* a, unsigned long long* 
                                 unsigned long long* base, unsigned long long job, int mixed, void* stream);
 int erik_launch_dmax(const double* D, int nD, int nbf, int nsh, const int* sh_bf0, const int* sh_n,
                      double* Dmax, void* stream);
+// integer shadows of the primitive pairs of all shell pairs; org: the atoms' integer positions, units of 2^-pu
+int erik_launch_prim_fx(const struct ShellPair* pairs, int npair, const struct PrimPair* prims, const int* sh_atom,
+                        const int64_t* org, int pu, struct PrimFx* out, void* stream);
 int erik_launch_symmetrize(double* M, int nD, int nbf, void* stream);
 int erik_launch_symcheck(const double* D, int nD, int nbf, unsigned long long* out, void* stream);
 int erik_launch_rys(int N, int n, const double* T, double* u, double* w, const int64_t* coef,

@@ -828,6 +828,7 @@ struct eri_plan {
   PrimPair* d_prims = nullptr;
   PrimPairF* d_primsf = nullptr;
   PrimFx* d_prfx = nullptr;
+  int64_t* d_org = nullptr;          // the atoms' integer positions
   int pu = 0;                        // unit 2^-pu of PrimFx::P
   bool fx_ok = true;                 // the FP32 launches may take the integer scalars
   bool fx64 = true;                  // the FP64 launches too: positions in units of 2^-SX_PU or finer
@@ -1013,12 +1014,12 @@ eri_status validate_basis(const eri_basis* b) {
 }
 
 
-// Integer shadows of the primitive pairs (eri_scalar.cuh): positions from a point near the
-// molecule's middle in units of 2^-pu that hold every P - Q in 60 bits.  One atom far away makes the
+// Unit of the integer shadows' positions (eri_scalar.cuh) and the atoms in it: from a point near the
+// molecule's middle, in units of 2^-pu that hold every P - Q in 60 bits.  One atom far away makes the
 // unit coarse for all: from SX_PU places on the FP64 launches take it, and the FP32 launches, which
-// round P - Q to 2^-24, from SX_PU32 on.  The exponents' range and the unit's lower end keep every
-// FP32 value made from them normal: T below 2^119, P - Q in units of 2^-99.
-void make_prim_fx(eri_plan* p, PrimFx* out) {
+// round P - Q to 2^-24, from SX_PU32 on.  The exponents' range (fx_range) and the unit's lower end keep
+// every FP32 value made from them normal: T below 2^119, P - Q in units of 2^-99.
+std::vector<int64_t> fx_positions(eri_plan* p) {
   double lo[3], hi[3], mid[3], ext = 0.0;
   for (int x = 0; x < 3; ++x) {
     lo[x] = hi[x] = p->coords[x];
@@ -1030,41 +1031,19 @@ void make_prim_fx(eri_plan* p, PrimFx* out) {
     ext = std::max(ext, std::max(hi[x] - mid[x], mid[x] - lo[x]));
     p->diag2 += (hi[x] - lo[x]) * (hi[x] - lo[x]);
   }
-  int e = 0;
+  int e = -40;
   if (ext > 0x1p-41) (void)std::frexp(std::min(2.0 * ext, 0x1p60), &e);   // |P - Q| <= 2 ext < 2^e
-  else e = -40;
   p->pu = 59 - e;
-  p->fx_ok = p->pu >= SX_PU32;
-  const double upu = p->fx_ok ? sx_pow2(p->pu) : 0.0;
+  p->fx_ok = p->fx_ok && p->pu >= SX_PU32;
+  p->fx64 = p->fx_ok && p->pu >= SX_PU;
   std::vector<int64_t> org(3 * p->natm, 0);
   if (p->fx_ok)
-    for (int k = 0; k < 3 * p->natm; ++k) org[k] = std::llrint((p->coords[k] - mid[k % 3]) * upu);
-  for (const ShellPair& sp : p->pairs_all)
-    for (int k = sp.prim_off; k < sp.prim_off + sp.nprim; ++k) {
-      const PrimPair& q = p->prims[k];
-      PrimFx& f = out[k];
-      memset(&f, 0, sizeof(f));
-      if (!(q.zeta > 1e-18 && q.zeta < 1e18) || !std::isfinite(q.E)) {
-        p->fx_ok = false;
-        continue;
-      }
-      f.H = 2.0 * q.hz;
-      const double root = std::sqrt(f.H);
-      f.E = q.E * root;
-      sx_from_double(f.H, &f.Hm, &f.He);
-      sx_from_double(root, &f.Sm, &f.Se);
-      double pa = 0.0;
-      for (int x = 0; x < 3; ++x) pa = std::max(pa, std::fabs(q.PA[x]));
-      int64_t m;
-      sx_from_double(1.0001 * (pa + 2.3507 * root), &m, &f.a);
-      const double u60 = sx_pow2(60 - f.a);
-      f.hz = std::llrint(q.hz * u60 * sx_pow2(-f.a));
-      for (int x = 0; x < 3; ++x) {
-        f.PA[x] = std::llrint(q.PA[x] * u60);
-        if (p->fx_ok) f.P[x] = org[3 * p->sh_atom[sp.sh0] + x] + std::llrint(q.PA[x] * upu);
-      }
-    }
+    for (int k = 0; k < 3 * p->natm; ++k) org[k] = std::llrint((p->coords[k] - mid[k % 3]) * sx_pow2(p->pu));
+  return org;
 }
+
+// Whether a primitive pair is in the integers' range.
+bool fx_range(const PrimPair& q) { return q.zeta > 1e-18 && q.zeta < 1e18 && std::isfinite(q.E); }
 
 // ---------------------------------------------------------------- J/K launch machinery
 struct Launch {
@@ -1414,7 +1393,7 @@ eri_status eri_plan_destroy(eri_plan* p) {
   if (p->side) cudaStreamDestroy(p->side);
   if (p->ev_fork) cudaEventDestroy(p->ev_fork);
   if (p->ev_join) cudaEventDestroy(p->ev_join);
-  void* bufs[] = {p->d_pairs_all, p->d_pairs, p->d_prims, p->d_primsf, p->d_prfx, p->d_sh_bf0, p->d_sh_n, p->d_sh_atom, p->d_Dmax, p->d_counters,
+  void* bufs[] = {p->d_pairs_all, p->d_pairs, p->d_prims, p->d_primsf, p->d_prfx, p->d_org, p->d_sh_bf0, p->d_sh_n, p->d_sh_atom, p->d_Dmax, p->d_counters,
                   p->d_stats, p->d_scratch, p->d_tasks, p->d_out, p->d_off, p->d_host_io, p->d_tlist,
                   p->d_tcount, p->d_tiles, p->d_gstats, p->d_symchk, p->d_err};
   for (void* b : bufs)
@@ -1545,6 +1524,7 @@ eri_status eri_plan_create(const eri_basis* basis, const eri_opts* opts, void* c
       pp.E = pref / pp.zeta * std::exp(-al * be / pp.zeta * AB2) * ca * cb;
       pp.hz = 0.5 / pp.zeta;
       pp.alpha = al;
+      p->fx_ok = p->fx_ok && fx_range(pp);
       p->prims.push_back(pp);
     }
     p->pairs_all.push_back(sp);
@@ -1561,6 +1541,7 @@ eri_status eri_plan_create(const eri_basis* basis, const eri_opts* opts, void* c
       cudaMalloc(&p->d_prims, sizeof(PrimPair) * p->prims.size()) != cudaSuccess ||
       cudaMalloc(&p->d_primsf, sizeof(PrimPairF) * p->prims.size()) != cudaSuccess ||
       cudaMalloc(&p->d_prfx, sizeof(PrimFx) * p->prims.size()) != cudaSuccess ||
+      cudaMalloc(&p->d_org, sizeof(int64_t) * 3 * p->natm) != cudaSuccess ||
       cudaMalloc(&p->d_sh_bf0, sizeof(int) * p->nshell) != cudaSuccess ||
       cudaMalloc(&p->d_sh_n, sizeof(int) * p->nshell) != cudaSuccess ||
       cudaMalloc(&p->d_sh_atom, sizeof(int) * p->nshell) != cudaSuccess ||
@@ -1592,13 +1573,13 @@ eri_status eri_plan_create(const eri_basis* basis, const eri_opts* opts, void* c
     f.pad[0] = f.pad[1] = 0.f;
   }
   PLAN_TRY(cudaMemcpyAsync(p->d_primsf, primsf.data(), sizeof(PrimPairF) * primsf.size(), cudaMemcpyHostToDevice, st));
-  std::vector<PrimFx> prfx(p->prims.size());
-  make_prim_fx(p, prfx.data());
-  p->fx64 = p->fx_ok && p->pu >= SX_PU;
-  PLAN_TRY(cudaMemcpyAsync(p->d_prfx, prfx.data(), sizeof(PrimFx) * prfx.size(), cudaMemcpyHostToDevice, st));
   PLAN_TRY(cudaMemcpyAsync(p->d_sh_bf0, p->sh_bf0.data(), sizeof(int) * p->nshell, cudaMemcpyHostToDevice, st));
   PLAN_TRY(cudaMemcpyAsync(p->d_sh_n, sh_n.data(), sizeof(int) * p->nshell, cudaMemcpyHostToDevice, st));
   PLAN_TRY(cudaMemcpyAsync(p->d_sh_atom, p->sh_atom.data(), sizeof(int) * p->nshell, cudaMemcpyHostToDevice, st));
+  const std::vector<int64_t> org = fx_positions(p);
+  PLAN_TRY(cudaMemcpyAsync(p->d_org, org.data(), sizeof(int64_t) * org.size(), cudaMemcpyHostToDevice, st));
+  if (p->fx_ok)
+    PLAN_TRY(erik_launch_prim_fx(p->d_pairs_all, (int)npair, p->d_prims, p->d_sh_atom, p->d_org, p->pu, p->d_prfx, st));
   PLAN_TRY(cudaMemsetAsync(p->d_stats, 0, sizeof(unsigned long long) * 4 * 256, st));
   PLAN_TRY(cudaMemsetAsync(p->d_err, 0, sizeof(unsigned), st));
 

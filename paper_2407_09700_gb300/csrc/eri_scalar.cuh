@@ -218,16 +218,16 @@ __device__ __forceinline__ void sx_root(const int64_t* __restrict__ coef, const 
 }
 #endif
 
-// 2^k for -1022 <= k <= 1023 (host)
-inline double sx_pow2(int k) {
+// 2^k for -1022 <= k <= 1023
+SX_HD double sx_pow2(int k) {
   const uint64_t u = (uint64_t)(k + 1023) << 52;
   double d;
   __builtin_memcpy(&d, &u, 8);
   return d;
 }
 
-// Mantissa and exponent of a normal v > 0, v = m 2^(e - 62), 2^61 <= m < 2^62 (host, exact).
-inline void sx_from_double(double v, int64_t* m, int* e) {
+// Mantissa and exponent of a normal v > 0, v = m 2^(e - 62), 2^61 <= m < 2^62 (exact).
+SX_HD void sx_from_double(double v, int64_t* m, int* e) {
   uint64_t u;
   __builtin_memcpy(&u, &v, 8);
   *e = (int)(u >> 52) - 1022;
