@@ -9,9 +9,9 @@
 // c_7 in units of 2^(E - 56) in the high and E in the low half of the last word, with
 // sum |c_k| < 2^E, so every partial sum fits 63 bits.  x in [-1, 1) is two's complement in units
 // of 2^-60: a signed top word (2^-31) and 29 low bits.  A step drops the product of the low
-// halves and the bits below 2^(E - 62), so the sums are off by less than 2^(E - 58) and the
-// value by that and the rounding of its conversion (worst relative error 1.2e-16 against the
-// polynomials, 1.15e-16 with FP64 sums).
+// halves and the lowest two bits of the sum, so the sums are off by at most 72 units of 2^(E - 62), 32 of
+// them from c_7 (44 seen), and the value by that and the rounding of its conversion (worst relative
+// error 1.2e-16 against the polynomials, 1.15e-16 with FP64 sums).
 #pragma once
 #include <stdint.h>
 
