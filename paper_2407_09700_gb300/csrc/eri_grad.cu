@@ -21,11 +21,15 @@
 //      Gamma_K = -w (D_ac D_bd + D_ad D_bc), w the permutation weight of the unique quartet
 //      (8 w ordered quartets share it); the 18 per-lane sums (J, K x centres A, B, C x xyz)
 //      are reduced over the team and 24 values (with D = -(A + B + C)) go to the gradient
-//      by FP64 atomics, once per quartet (Alg. 4's accumulate-then-add).
+//      by FP64 atomics, once per quartet or range (Alg. 4's accumulate-then-add), each team to
+//      one of 32 copies that are added pairwise at the end.  With one copy the additions of split
+//      quartets' ranges left errors of 6.2e-15, 4.3e-15 and 5.7e-15 in gradients of 3, 5 and 6
+//      atoms (2.3e-15, 3.6e-15, 3.5e-15 unsplit), with 32 they leave 1.5e-15, 1.3e-15, 1.3e-15,
+//      and the teams wait less for one another (5 atoms 4.68 -> 3.17 ms).
 // Everything runs in FP64.  A class whose candidate quartets cannot fill the grid splits each into
 // ranges of its primitive quartets and one of few candidates screens in the kernel, as in the J/K
 // build (every step after the contraction is linear in the contracted sets): gradient of 5 atoms
-// with 6-31G(d)-like shells 14.7 -> 5.2 ms, of 4 atoms with s..g shells 248 -> 199 ms.
+// with 6-31G(d)-like shells 14.7 -> 4.7 ms, of 4 atoms with s..g shells 248 -> 173 ms.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -520,16 +524,18 @@ __global__ void __launch_bounds__(TPB, (TS == 1 ? 3 : 2)) eri_grad_kernel(const 
     if (active && tl == 0) {
       const int atA = __ldg(ga.sh_atom + bra->sh0), atB = __ldg(ga.sh_atom + bra->sh1);
       const int atC = __ldg(ga.sh_atom + ket->sh0), atD = __ldg(ga.sh_atom + ket->sh1);
+      double* gJ = ga.sum + (size_t)(gteam % GRAD_COPIES) * 6 * ga.natm;
+      double* gK = gJ + 3 * ga.natm;
 #pragma unroll
       for (int x = 0; x < 3; ++x) {
-        atomicAdd(ga.gJ + 3 * atA + x, jA[x]);
-        atomicAdd(ga.gJ + 3 * atB + x, jB[x]);
-        atomicAdd(ga.gJ + 3 * atC + x, jC[x]);
-        atomicAdd(ga.gJ + 3 * atD + x, -(jA[x] + jB[x] + jC[x]));
-        atomicAdd(ga.gK + 3 * atA + x, kA[x]);
-        atomicAdd(ga.gK + 3 * atB + x, kB[x]);
-        atomicAdd(ga.gK + 3 * atC + x, kC[x]);
-        atomicAdd(ga.gK + 3 * atD + x, -(kA[x] + kB[x] + kC[x]));
+        atomicAdd(gJ + 3 * atA + x, jA[x]);
+        atomicAdd(gJ + 3 * atB + x, jB[x]);
+        atomicAdd(gJ + 3 * atC + x, jC[x]);
+        atomicAdd(gJ + 3 * atD + x, -(jA[x] + jB[x] + jC[x]));
+        atomicAdd(gK + 3 * atA + x, kA[x]);
+        atomicAdd(gK + 3 * atB + x, kB[x]);
+        atomicAdd(gK + 3 * atC + x, kC[x]);
+        atomicAdd(gK + 3 * atD + x, -(kA[x] + kB[x] + kC[x]));
       }
     }
     team_sync<TS>();
@@ -542,6 +548,16 @@ __global__ void __launch_bounds__(TPB, (TS == 1 ? 3 : 2)) eri_grad_kernel(const 
     atomicAdd(a.stats + 0, cnt_q);
     atomicAdd(a.stats + 1, cnt_p);
   }
+}
+
+// A warp per value: lane c reads copy c, the warp adds them pairwise.
+__global__ void grad_sum_kernel(const double* sum, int natm, double* gJ, double* gK) {
+  static_assert(GRAD_COPIES == 32, "a lane per copy");
+  const int v = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), n = 3 * natm;
+  if (v >= 2 * n) return;
+  double t = sum[(size_t)(threadIdx.x & 31) * 2 * n + v];
+  for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+  if ((threadIdx.x & 31) == 0) *(v < n ? gJ + v : gK + v - n) = t;
 }
 
 // ------------------------------------------------------------------ host launchers
@@ -574,5 +590,10 @@ extern "C" int erik_launch_grad(int ts, const GradArgs* a, int grid, int smem_by
     case 128: eri_grad_kernel<128><<<grid, TPB, smem_bytes, s>>>(*a); break;
     default: return (int)cudaErrorInvalidValue;
   }
+  return (int)cudaGetLastError();
+}
+
+extern "C" int erik_launch_grad_sum(const double* sum, int natm, double* gJ, double* gK, void* stream) {
+  grad_sum_kernel<<<(6 * natm + 3) / 4, TPB, 0, (cudaStream_t)stream>>>(sum, natm, gJ, gK);
   return (int)cudaGetLastError();
 }

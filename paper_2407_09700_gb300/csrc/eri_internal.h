@@ -224,9 +224,11 @@ struct GradArgs {
   KernelArgs k;          // task space, pair data, compacted list, Rys table of nroots
   GradDesc g;
   const int* sh_atom;    // [nshell] atom of each shell
-  double* gJ;            // [natm][3] += d E_J / d R
-  double* gK;            // [natm][3] += d E_K / d R
+  double* sum;           // [GRAD_COPIES][2][natm][3] += d E_J / d R, d E_K / d R: teams add to the copies in turn
+  int natm;
 };
+// Copies of the gradient that the teams of eri_jk_grad add to.
+#define GRAD_COPIES 32
 
 // Host-side launchers implemented in eri_kernels.cu.  All return a cudaError_t as int.
 #ifdef __cplusplus
@@ -274,6 +276,8 @@ int erik_launch_fixed(int ts, int tiles, const struct KernelArgs* a, int grid, i
 int erik_upload_cart_tables_grad(void);
 int erik_grad_blocks_per_sm(int ts, int smem_bytes, int* out);
 int erik_launch_grad(int ts, const struct GradArgs* a, int grid, int smem_bytes, void* stream);
+// gJ, gK [natm][3] = the sum of the copies
+int erik_launch_grad_sum(const double* sum, int natm, double* gJ, double* gK, void* stream);
 #ifdef __cplusplus
 }
 #endif

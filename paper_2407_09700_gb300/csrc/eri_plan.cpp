@@ -852,6 +852,7 @@ struct eri_plan {
   unsigned long long* d_tcount = nullptr;     // [256][2] FP64 / FP32 list lengths
   unsigned* d_tiles = nullptr;                // per-tile counts / offsets of the compaction
   unsigned long long* d_gstats = nullptr;     // [2] quartets / primitive quartets of eri_jk_grad
+  double* d_gsum = nullptr;                   // the copies of the gradient that its teams add to
   unsigned long long* d_symchk = nullptr;     // [2] max|D_ij - D_ji|, max|D| (check_symmetric)
   unsigned* d_err = nullptr;                  // set by a kernel whose bounded device wait gave up
   cudaStream_t grad_stream = nullptr;
@@ -1395,7 +1396,7 @@ eri_status eri_plan_destroy(eri_plan* p) {
   if (p->ev_join) cudaEventDestroy(p->ev_join);
   void* bufs[] = {p->d_pairs_all, p->d_pairs, p->d_prims, p->d_primsf, p->d_prfx, p->d_org, p->d_sh_bf0, p->d_sh_n, p->d_sh_atom, p->d_Dmax, p->d_counters,
                   p->d_stats, p->d_scratch, p->d_tasks, p->d_out, p->d_off, p->d_host_io, p->d_tlist,
-                  p->d_tcount, p->d_tiles, p->d_gstats, p->d_symchk, p->d_err};
+                  p->d_tcount, p->d_tiles, p->d_gstats, p->d_gsum, p->d_symchk, p->d_err};
   for (void* b : bufs)
     if (b) cudaFree(b);
   delete p;
@@ -1707,14 +1708,15 @@ eri_status eri_jk_grad(eri_plan* p, const double* D, double* gJ, double* gK, voi
   if ((s = ensure_buf(&p->d_tlist, &p->tlist_cap, 2 * maxnt)) != ERI_OK) return s;
   if ((s = ensure_buf(&p->d_tiles, &p->tiles_cap, 2 * tiles)) != ERI_OK) return s;
   if (!p->d_gstats) CUDA_TRY(cudaMalloc(&p->d_gstats, sizeof(unsigned long long) * 2));
+  const size_t gsum_bytes = sizeof(double) * 6 * GRAD_COPIES * (size_t)p->natm;
+  if (!p->d_gsum) CUDA_TRY(cudaMalloc(&p->d_gsum, gsum_bytes));
   if (!p->side) {
     CUDA_TRY(cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking));
     CUDA_TRY(cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming));
     CUDA_TRY(cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming));
   }
   const cudaStream_t ss[2] = {st, p->side};
-  CUDA_TRY(cudaMemsetAsync(gJ, 0, sizeof(double) * 3 * p->natm, st));
-  CUDA_TRY(cudaMemsetAsync(gK, 0, sizeof(double) * 3 * p->natm, st));
+  CUDA_TRY(cudaMemsetAsync(p->d_gsum, 0, gsum_bytes, st));
   CUDA_TRY(cudaMemsetAsync(p->d_gstats, 0, sizeof(unsigned long long) * 2, st));
   CUDA_TRY(erik_launch_dmax(D, 1, p->nbf, p->nshell, p->d_sh_bf0, p->d_sh_n, p->d_Dmax, st));
   CUDA_TRY(cudaMemsetAsync(p->d_counters, 0, sizeof(unsigned long long) * 256, st));
@@ -1765,13 +1767,14 @@ eri_status eri_jk_grad(eri_plan* p, const double* D, double* gJ, double* gK, voi
     ga.k = a;
     ga.g = g;
     ga.sh_atom = p->d_sh_atom;
-    ga.gJ = gJ;
-    ga.gK = gK;
+    ga.sum = p->d_gsum;
+    ga.natm = p->natm;
     CUDA_TRY(erik_launch_grad(l.ts, &ga, l.grid, l.smem, sl));
     ++li;
   }
   CUDA_TRY(cudaEventRecord(p->ev_join, p->side));
   CUDA_TRY(cudaStreamWaitEvent(st, p->ev_join, 0));
+  CUDA_TRY(erik_launch_grad_sum(p->d_gsum, p->natm, gJ, gK, st));
   p->grad_stream = st;
   return ERI_OK;
 }
