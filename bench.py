@@ -288,11 +288,11 @@ def rys_model_flops(r, nD=1):
 
 def kernel_name(r):
     prec = "float" if r["fp32"] else "double"
-    if r["specialised"] and not r["fp32"]:      # the workloads' exponents are in the integers' range
+    if r["kernel"] == "small_fx":
         return f"eri_small_fx_kernel<{r['la']}, {r['lb']}, {r['lc']}, {r['ld']}>"
-    if r["specialised"]:
+    if r["kernel"] == "small":
         return f"eri_small_kernel<{r['la']}, {r['lb']}, {r['lc']}, {r['ld']}, {prec}>"
-    if not r["fp32"] and r["la"] + r["lb"] + r["lc"] + r["ld"] <= 8 and r["team_size"] in (16, 32):
+    if r["kernel"] == "fixed":
         return f"eri_fixed_kernel<{r['team_size']}>"
     xy = "true" if r["shared_products"] else "false"
     if r.get("compiled_class"):

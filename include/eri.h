@@ -260,6 +260,15 @@ eri_status eri_set_profiling(eri_plan* plan, int enable);
  * out (HOST) and the number available to *n.  Requires profiling to have been on. */
 eri_status eri_launch_records(eri_plan* plan, eri_launch_record* out, int cap, int* n);
 
+/* Kernel of a launch: the general class kernel, the specialised one-lane kernel in floating
+ * point or in integer arithmetic (FP64 launches), and the class kernel with the fixed-point sums of
+ * Eq. 1 (FP64 launches of s, p and d classes). */
+enum { ERI_KERNEL_CLASS = 0, ERI_KERNEL_SMALL = 1, ERI_KERNEL_SMALL_FX = 2, ERI_KERNEL_FIXED = 3 };
+
+/* Kernels of the launches of the last recorded call, in the order of eri_launch_records: writes up to
+ * cap values to out (HOST) and the number available to *n. */
+eri_status eri_launch_kernels(const eri_plan* plan, int* out, int cap, int* n);
+
 /*
  * Batched J/K over several jobs (the serving pattern): every job is (plan, D, J, K,
  * flags) exactly as for eri_jk, and the result of each job is that of eri_jk on it

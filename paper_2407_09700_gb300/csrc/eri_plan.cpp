@@ -870,7 +870,7 @@ struct eri_plan {
   bool profiling = false;
   std::vector<cudaEvent_t> events;            // 2 per launch
   std::vector<int> last_launch_xy;            // X*15+Y per launch
-  std::vector<int> last_launch_ts, last_launch_grid, last_launch_fp32, last_launch_small, last_launch_fixed;
+  std::vector<int> last_launch_ts, last_launch_grid, last_launch_fp32, last_launch_kernel;
   std::vector<int> last_launch_qsplit, last_launch_listed;
 };
 
@@ -1249,8 +1249,7 @@ eri_status run_jk(eri_plan* p, const std::vector<Launch>& launches, const double
   p->last_launch_ts.clear();
   p->last_launch_grid.clear();
   p->last_launch_fp32.clear();
-  p->last_launch_small.clear();
-  p->last_launch_fixed.clear();
+  p->last_launch_kernel.clear();
   p->last_launch_qsplit.clear();
   p->last_launch_listed.clear();
   if (nstreams == 2) {
@@ -1308,8 +1307,7 @@ eri_status run_jk(eri_plan* p, const std::vector<Launch>& launches, const double
       p->last_launch_ts.push_back(l.ts);
       p->last_launch_grid.push_back(l.grid);
       p->last_launch_fp32.push_back(l.fp32);
-      p->last_launch_small.push_back(l.small ? 1 : 0);
-      p->last_launch_fixed.push_back(l.fixed);
+      p->last_launch_kernel.push_back(l.small == 2 ? ERI_KERNEL_SMALL_FX : (l.small ? ERI_KERNEL_SMALL : (l.fixed ? ERI_KERNEL_FIXED : ERI_KERNEL_CLASS)));
       p->last_launch_qsplit.push_back(l.qsplit);
       p->last_launch_listed.push_back(listed ? 1 : 0);
     }
@@ -1986,13 +1984,22 @@ eri_status eri_launch_records(eri_plan* p, eri_launch_record* out, int cap, int*
     r.model_flops = (a64 + a32) * (double)r.prim_quartets + (q64 + q32) * (double)r.quartets;
     r.model_flops_fp32 = a32 * (double)r.prim_quartets + q32 * (double)r.quartets;
     r.fp32 = f;
-    r.specialised = p->last_launch_small[i];
-    const bool cls64 = !f && !r.specialised && !p->last_launch_fixed[i];
+    const int kernel = p->last_launch_kernel[i];
+    r.specialised = (kernel == ERI_KERNEL_SMALL || kernel == ERI_KERNEL_SMALL_FX) ? 1 : 0;
+    const bool cls64 = !f && kernel == ERI_KERNEL_CLASS;
     r.shared_products = (cls64 && c.xy) ? 1 : 0;
     r.compiled_class = (cls64 && erik_class_spec_available(r.team_size, c.la, c.lb, c.lc, c.ld)) ? 1 : 0;
     r.quartet_split = p->last_launch_qsplit[i];
     r.listed = p->last_launch_listed[i];
   }
+  return ERI_OK;
+}
+
+eri_status eri_launch_kernels(const eri_plan* p, int* out, int cap, int* n) {
+  g_err.clear();
+  if (!p || !n || (cap > 0 && !out)) return fail(ERI_ERR_ARG, "NULL argument");
+  *n = (int)p->last_launch_kernel.size();
+  for (int i = 0; i < *n && i < cap; ++i) out[i] = p->last_launch_kernel[i];
   return ERI_OK;
 }
 

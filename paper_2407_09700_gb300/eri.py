@@ -20,6 +20,7 @@ ERI_OK, ERI_ERR_ARG, ERI_ERR_BASIS, ERI_ERR_OOM, ERI_ERR_CUDA, ERI_ERR_NO_DEVICE
     ERI_ERR_UNSUPPORTED_L = range(8)
 ERI_FP64, ERI_MIXED = 0, 1
 ERI_WANT_J, ERI_WANT_K = 1, 2
+LAUNCH_KERNELS = ("class", "small", "small_fx", "fixed")      # ERI_KERNEL_*
 
 _dp = ctypes.POINTER(ctypes.c_double)
 _ip = ctypes.POINTER(ctypes.c_int)
@@ -86,6 +87,7 @@ _SIGS = {
     "eri_set_profiling": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int]),
     "eri_launch_records": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(eri_launch_record), ctypes.c_int,
                                           ctypes.POINTER(ctypes.c_int)]),
+    "eri_launch_kernels": (ctypes.c_int, [ctypes.c_void_p, _ip, ctypes.c_int, _ip]),
     "eri_one_electron": (ctypes.c_int, [ctypes.POINTER(eri_basis), ctypes.c_int, _dp, _dp, _dp, _dp, _dp]),
     "eri_batch_create": (ctypes.c_int, [ctypes.POINTER(ctypes.c_void_p)]),
     "eri_batch_destroy": (ctypes.c_int, [ctypes.c_void_p]),
@@ -260,11 +262,14 @@ class Plan:
         _check(load_library().eri_set_profiling(self._h, 1 if on else 0))
 
     def launch_records(self):
-        """Per-launch records of the last jk call (class, team size, ms, counts, model FLOPs)."""
+        """Per-launch records of the last jk call (class, team size, ms, counts, model FLOPs, kernel)."""
         arr = (eri_launch_record * 256)()
         n = ctypes.c_int()
         _check(load_library().eri_launch_records(self._h, arr, 256, ctypes.byref(n)))
-        return [{k: getattr(arr[i], k) for k, _ in eri_launch_record._fields_} for i in range(n.value)]
+        kern = (ctypes.c_int * 256)()
+        _check(load_library().eri_launch_kernels(self._h, kern, 256, ctypes.byref(n)))
+        return [{**{k: getattr(arr[i], k) for k, _ in eri_launch_record._fields_}, "kernel": LAUNCH_KERNELS[kern[i]]}
+                for i in range(n.value)]
 
     def stats(self):
         s = eri_stats()
