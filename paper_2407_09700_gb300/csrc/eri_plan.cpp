@@ -817,7 +817,7 @@ struct eri_plan {
   int type_maxprim[ERI_NPAIRTYPE] = {0};   // most primitive pairs of a kept pair, per type
   long long type_sumprim[ERI_NPAIRTYPE] = {0};   // primitive pairs of the kept pairs, per type
   double type_spread[ERI_NPAIRTYPE] = {0}; // (l0 + l1) / 2 log2 of the largest ratio of a kept pair's zeta
-  double type_rt[ERI_NPAIRTYPE] = {0};     // l0 + l1 > 0: bound of zeta |P - Q|^2 over the kept pairs' primitives
+  double type_rt[ERI_NPAIRTYPE] = {0};     // l0 + l1 > 0: bound of zeta |P - Q|^2 over the kept pairs (fx_zeta)
   double diag2 = 0.0;                // squared diagonal of the atoms' bounding box
   int npairs_kept = 0;
   std::vector<double> Q;             // [nshell*nshell]
@@ -1041,6 +1041,21 @@ std::vector<int64_t> fx_positions(eri_plan* p) {
   if (p->fx_ok)
     for (int k = 0; k < 3 * p->natm; ++k) org[k] = std::llrint((p->coords[k] - mid[k % 3]) * sx_pow2(p->pu));
   return org;
+}
+
+// zeta of the bound SX_TMAX for one pair: the largest or, if that is above the bound, the one that stands for
+// the contracted pair.  Its primitives leave errors like E / sqrt(zeta) (the unit of C) in values like
+// E / zeta (C), so a contracted core shell beside a valence p shell counts as its diffuse primitives do.
+double fx_zeta(const eri_plan* p, const ShellPair& sp, double zmax) {
+  if (zmax * p->diag2 <= SX_TMAX) return zmax;
+  double err = 0.0, val = 0.0;
+  for (int k = sp.prim_off; k < sp.prim_off + sp.nprim; ++k) {
+    const PrimPair& q = p->prims[k];
+    err += std::fabs(q.E) * std::sqrt(q.hz);
+    val += std::fabs(q.E) * q.hz;
+  }
+  const double r = err / val;                       // sqrt(2 zeta)
+  return r > 0.0 ? std::min(zmax, 0.5 * r * r) : zmax;
 }
 
 // Whether a primitive pair is in the integers' range.
@@ -1632,7 +1647,7 @@ eri_status eri_plan_create(const eri_basis* basis, const eri_opts* opts, void* c
         // unsorted, a batch of a mixed plan holds exponents further apart: 6 binades less allowed
         const double spread = 0.5 * (p->sh_l[sp.sh0] + p->sh_l[sp.sh1]) * std::log2(zhi / zlo);
         p->type_spread[X] = std::max(p->type_spread[X], spread + (p->opts.precision == ERI_MIXED ? 6.0 : 0.0));
-        if (p->sh_l[sp.sh0] > 0) p->type_rt[X] = std::max(p->type_rt[X], zhi * p->diag2);
+        if (p->sh_l[sp.sh0] > 0) p->type_rt[X] = std::max(p->type_rt[X], fx_zeta(p, sp, zhi) * p->diag2);
       }
     }
     p->type_cnt[X] = (int)kept.size() - p->type_off[X];

@@ -93,3 +93,21 @@ def test_range_of_the_integer_kernel(zeta, R, ss, ps):
     Jr, Kr, _ = oracle.jk(m, tau=0.0)
     for got, ref in ((J, Jr), (K, Kr)):
         assert np.abs(got - ref).max() <= 2e-14 * np.abs(ref).max()
+
+
+# A contracted core s shell (exponents up to 2e4) beside a p shell counts as its diffuse primitives: the integer
+# kernel serves it, and the dipole (px s| in the field of an s function 8 bohr away, where P = A is exact in
+# the oracle too, is as close as that of the single exponents.
+def test_contracted_core_stays_in_integers():
+    core = np.array([2e4, 3e3, 600.0, 150.0, 40.0, 10.0])
+    one = np.ones(1)
+    m = custom_molecule(np.array([[0.0, 0, 0], [8.0, 0, 0]]),
+                        [(0, 0, core, np.array([0.002, 0.015, 0.07, 0.22, 0.47, 0.36])),
+                         (0, 1, np.array([8.0, 2.0]), np.array([0.4, 0.7])), (1, 0, np.array([0.5]), one)])
+    m.D = np.zeros((1, m.nbf, m.nbf))
+    m.D[0, -1, -1] = 1.0
+    J, _, kern = _jk(m)
+    assert kern[1, 0, 0, 0] == "small_fx" and kern[1, 0, 1, 0] == "small_fx"
+    Jr, _, _ = oracle.jk(m, tau=0.0)
+    for at in ((0, 0), (0, 1), (1, 1)):
+        assert abs(J[0][at] / Jr[0][at] - 1) <= 8e-15
