@@ -294,19 +294,6 @@ const void* fixed_ptr(int ts, int tiles) {
 
 extern "C" int erik_upload_cart_tables_fixed(void) { return (int)upload_cart_table(); }
 
-// Instantiation i (0, 1, ...) to *ts and *tiles; 0 past the last one.
-extern "C" int erik_fixed_variant(int i, int* ts, int* tiles) {
-  static const int v[][2] = {
-#define FIXED_ROW(T, NT) {T, NT},
-      FIXED_KERNELS(FIXED_ROW)
-#undef FIXED_ROW
-  };
-  if (i < 0 || i >= (int)(sizeof(v) / sizeof(v[0]))) return 0;
-  *ts = v[i][0];
-  *tiles = v[i][1];
-  return 1;
-}
-
 extern "C" int erik_fixed_blocks_per_sm(int ts, int tiles, int smem_bytes, int* out) {
   const void* k = fixed_ptr(ts, tiles);
   if (!k) return (int)cudaErrorInvalidValue;

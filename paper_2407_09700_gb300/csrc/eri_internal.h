@@ -266,10 +266,8 @@ int erik_launch_small(int la, int lb, int lc, int ld, int fp32, const struct Ker
 // the FP64 launches of these classes in integer arithmetic
 int erik_small_fx_blocks_per_sm(int la, int lb, int lc, int ld, int* out);
 int erik_launch_small_fx(int la, int lb, int lc, int ld, const struct KernelArgs* a, int grid, void* stream);
-// class kernels with the fixed-point assembly (eri_fixed.cu): instantiated lanes per quartet and
-// tiles per lane and pass
+// class kernels with the fixed-point assembly (eri_fixed.cu)
 int erik_upload_cart_tables_fixed(void);
-int erik_fixed_variant(int i, int* ts, int* tiles);
 int erik_fixed_blocks_per_sm(int ts, int tiles, int smem_bytes, int* out);
 int erik_launch_fixed(int ts, int tiles, const struct KernelArgs* a, int grid, int smem_bytes, void* stream);
 // energy-gradient class kernels (eri_grad.cu)

@@ -209,10 +209,10 @@ ClassTune class_tune(int la, int lb, int lc, int ld) {
 // split until every group size occurs a multiple of T times (a leftover group of size
 // s > 1 becomes s-1 and 1; a leftover of single values is padded) and dealt out so that
 // each lane of a T-lane team gets one group of each program entry.  Out: slot_val[o] =
-// value index or -1 (padding) for slot o = (k / G) * G T + (k % G) * T + lane of the
-// lane's k-th slot (G slots per pass); gm[pass] bit k % G set where slot k starts a group
-// (every pass starts one); *slots_per_lane.
-void lane_programs(const std::vector<int>& key, int T, int G, std::vector<int>* slot_val, std::vector<uint32_t>* gm,
+// value index or -1 (padding) for slot o = (k / 32) * 32 T + (k % 32) * T + lane of the
+// lane's k-th slot; gm[pass] bit k % 32 set where slot k starts a group (every pass starts
+// one); *slots_per_lane.
+void lane_programs(const std::vector<int>& key, int T, std::vector<int>* slot_val, std::vector<uint32_t>* gm,
                    int* slots_per_lane) {
   std::vector<std::pair<int, int>> kv;
   for (int v = 0; v < (int)key.size(); ++v) kv.push_back({key[v], v});
@@ -252,20 +252,20 @@ void lane_programs(const std::vector<int>& key, int T, int G, std::vector<int>* 
   }
   int Ls = 0;
   for (int sz : prog) Ls += sz;
-  const int npass = (Ls + G - 1) / G;
-  slot_val->assign((size_t)npass * G * T, -1);
+  const int npass = (Ls + 31) / 32;
+  slot_val->assign((size_t)npass * 32 * T, -1);
   slot_val->resize((size_t)Ls * T);
   gm->assign(npass, 0u);
   int k = 0;
   for (int sz : prog) {
-    (*gm)[k / G] |= 1u << (k % G);
+    (*gm)[k / 32] |= 1u << (k % 32);
     k += sz;
   }
   for (int p = 0; p < npass; ++p) (*gm)[p] |= 1u;
   for (int ln = 0; ln < T; ++ln) {
     int kk = 0;
     for (const auto& g : lane[ln])
-      for (size_t m = 0; m < g.size(); ++m, ++kk) (*slot_val)[(kk / G) * G * T + (kk % G) * T + ln] = g[m];
+      for (size_t m = 0; m < g.size(); ++m, ++kk) (*slot_val)[(kk / 32) * 32 * T + (kk % 32) * T + ln] = g[m];
   }
   *slots_per_lane = Ls;
 }
@@ -343,7 +343,7 @@ void make_class(int la, int lb, int lc, int ld, ClassDesc* c, int* ts, std::vect
     std::vector<int> sv;
     std::vector<uint32_t> gm;
     int Ls = 0;
-    lane_programs(key, T, 32, &sv, &gm, &Ls);
+    lane_programs(key, T, &sv, &gm, &Ls);
     c->nslot = Ls * T;
     c->npass = (int)gm.size();
     std::vector<uint32_t> outi(c->nslot, 1u << 31), dst(c->nslot, 0);
@@ -588,7 +588,7 @@ void make_grad_class(int la, int lb, int lc, int ld, GradDesc* g, int* ts, std::
   std::vector<int> sv;
   std::vector<uint32_t> gm;
   int Ls = 0;
-  lane_programs(key, *ts, 32, &sv, &gm, &Ls);
+  lane_programs(key, *ts, &sv, &gm, &Ls);
   g->nslot = Ls * *ts;
   g->npass = (int)gm.size();
   std::vector<uint32_t> dst(g->nslot, 0);
@@ -1492,12 +1492,12 @@ eri_status eri_plan_create(const eri_basis* basis, const eri_opts* opts, void* c
       // by total exponent: the fixed-point kernels scale batches of neighbours together
       // mixed plans keep the shells' order: the FP32 launches add their FP32 sums in it
       if (p->opts.precision != ERI_MIXED)
-      std::stable_sort(t.keep.begin(), t.keep.end(), [&](int c0, int c1) {
-        const int nb = p->sh_nprim[b];
-        const double z0 = p->exps[p->sh_off[a] + c0 / nb] + p->exps[p->sh_off[b] + c0 % nb];
-        const double z1 = p->exps[p->sh_off[a] + c1 / nb] + p->exps[p->sh_off[b] + c1 % nb];
-        return z0 < z1;
-      });
+        std::stable_sort(t.keep.begin(), t.keep.end(), [&](int c0, int c1) {
+          const int nb = p->sh_nprim[b];
+          const double z0 = p->exps[p->sh_off[a] + c0 / nb] + p->exps[p->sh_off[b] + c0 % nb];
+          const double z1 = p->exps[p->sh_off[a] + c1 / nb] + p->exps[p->sh_off[b] + c1 % nb];
+          return z0 < z1;
+        });
       t.np = (int)t.keep.size();
       tmp.push_back(std::move(t));
     }
@@ -2028,19 +2028,19 @@ eri_status eri_check_class_tables(int* nclasses, int* problems) {
   if (!nclasses || !problems) return fail(ERI_ERR_ARG, "NULL output");
   const CartTab& ct = cart();
   int bad = 0, n = 0;
-  auto check_lp = [&](const uint32_t* outi, const uint32_t* dst, const uint32_t* gm, int T, int G, int nslot, int nval,
+  auto check_lp = [&](const uint32_t* outi, const uint32_t* dst, const uint32_t* gm, int T, int nslot, int nval,
                       auto&& expect) {
     const int Ls = nslot / T;
     if (Ls * T != nslot) ++bad;
     std::vector<int> seen(nval, 0);
-    for (int p = 0; p < (Ls + G - 1) / G; ++p)
+    for (int p = 0; p < (Ls + 31) / 32; ++p)
       if (!(gm[p] & 1u)) ++bad;
     for (int ln = 0; ln < T; ++ln) {
       uint32_t cur = 0xffffffffu;
       for (int k = 0; k < Ls; ++k) {
-        const int o = (k / G) * T * G + (k % G) * T + ln;
+        const int o = (k / 32) * T * 32 + (k % 32) * T + ln;
         const uint32_t q = outi[o];
-        if ((gm[k / G] >> (k % G)) & 1u) cur = q & 0xffffu;
+        if ((gm[k / 32] >> (k % 32)) & 1u) cur = q & 0xffffu;
         if (q >> 31) continue;
         if ((q & 0xffffu) != cur) ++bad;
         if ((int)dst[o] < 0 || (int)dst[o] >= nval) { ++bad; continue; }
@@ -2067,7 +2067,7 @@ eri_status eri_check_class_tables(int* nclasses, int* problems) {
           return (uint32_t)(ct.lx[e] * L1 + ct.lx[f]) | ((uint32_t)(ct.ly[e] * L1 + ct.ly[f]) << 8) |
                  ((uint32_t)(ct.lz[e] * L1 + ct.lz[f]) << 16);
         };
-        check_lp(idx.data(), idx.data() + c.dst_off, idx.data() + c.gmask_off, ts, 32, c.nslot, c.nout,
+        check_lp(idx.data(), idx.data() + c.dst_off, idx.data() + c.gmask_off, ts, c.nslot, c.nout,
                  [&](int v, uint32_t q) { return (q & 0xffffffu) == word(v); });
         const int tpb = 128 / ts;
         if (ts > 1 && (8L * c.team_doubles * tpb > 200 * 1024 || 8L * c.team_doubles_f32 * tpb > 200 * 1024)) ++bad;
@@ -2130,7 +2130,7 @@ eri_status eri_check_class_tables(int* nclasses, int* problems) {
                  ((q >> 8) & 0xffu) == (uint32_t)(ct.ly[e] * L1 + ct.ly[f]) &&
                  ((q >> 16) & 0xfffu) == (uint32_t)(set * NnI + ct.lz[e] * L1 + ct.lz[f]);
         };
-        check_lp(idx.data(), idx.data() + g.dst_off, idx.data() + g.gmask_off, ts, 32, g.nslot, g.nout, expect);
+        check_lp(idx.data(), idx.data() + g.dst_off, idx.data() + g.gmask_off, ts, g.nslot, g.nout, expect);
         if (ts > 1 && 8L * g.team_doubles * (128 / ts) > 200 * 1024) ++bad;
       }
     }
