@@ -340,7 +340,9 @@ def roofline_of(per, peak64, peak32=None):
             "flops_kind": "achieved / frac: operations of the OS/HGP oracle (its instrumented counter per class, "
                           "tests/golden/oracle_class_ops.json) for the primitive and contracted quartets the "
                           "launches evaluated; model_*: the kernel's own operation count (FMA = 2); rys_model_*: "
-                          "the Rys-model count (roots, 2D tables, Eq. 1 at 3 FLOP per term, digestion)",
+                          "the Rys-model count (roots, 2D tables, Eq. 1 at 3 FLOP per term, digestion).  "
+                          "eri_fixed_kernel and eri_small_fx_kernel do part of these operations on the integer "
+                          "pipes: their fractions compare operation counts with the FP64 peak, not pipe use",
             "traffic_note": "null: pair data, D, J and K stay in L2 (DRAM bytes per launch do not grow with its "
                             "work; see profiles/)"}
 
@@ -392,7 +394,7 @@ def leg_mixed(pkg, mol, D, J64, K64, steps, flush, stream, table, peak64, peak32
            "mixed_thresh": MIXED_THRESH,
            "split": "FP32 recurrences where the transfer-aware bound Qe_ij Qe_kl max|D| <= mixed_thresh",
            "max_abs_dJ_vs_fp64": float((Jm - J64).abs().max()), "max_abs_dK_vs_fp64": float((Km - K64).abs().max()),
-           "fp64_pipe_frac": f64 / pt / 1e12 / peak64, "fp32_pipe_frac": f32 / pt / 1e12 / peak32,
+           "fp64_model_frac": f64 / pt / 1e12 / peak64, "fp32_model_frac": f32 / pt / 1e12 / peak32,
            "kernel_shares": shares_of(per)}
     plan_m.close()
     return out

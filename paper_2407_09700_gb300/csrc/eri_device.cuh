@@ -108,8 +108,8 @@ __device__ __forceinline__ void rys_root(const int64_t* __restrict__ coef, const
   }
 }
 
-// The same root and weight by Horner's rule in FP64, for kernels whose integer pipes are the busier
-// ones (eri_fixed.cu: (dp|pp) 54 ms against 61 ms with the fixed-point sums on the 16-atom build).
+// The same root and weight by Horner's rule in FP64, for eri_fixed.cu, where it is faster ((dp|pp) 54 ms
+// against 61 ms with the fixed-point sums on the 16-atom build: its integer pipes have Eq. 1 to do).
 __device__ __forceinline__ void rys_root64(const double* __restrict__ coef, const double* __restrict__ au,
                                            const double* __restrict__ aw, int N, const RysAt& at, int n, double& u,
                                            double& w) {

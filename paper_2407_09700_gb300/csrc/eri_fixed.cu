@@ -1,7 +1,8 @@
 // FP64-accurate class kernels with the Eq. 1 assembly in block fixed point (eri_fixed.cuh), for
 // the classes that run with more than one lane per shell quartet.  Teams, tasks, batches of
 // primitive quartets, the transfer relations and the digestion are those of eri_class_kernel
-// (see eri_kernels.cu); the roots, weights and 2D recurrences are FP64 as there.  Per batch:
+// (see eri_kernels.cu); the 2D recurrences are FP64 as there, the roots and weights FP64 Horner sums
+// (rys_root64: in 64-bit integers, as in the class kernel, (dp|pp) took 61 instead of 54 ms).  Per batch:
 //   a. primitive-quartet scalars, b. roots and 2D tables (FP64, in shared memory);
 //   c. lanes over the table entries: the largest exponent of the entry over the batch's
 //      primitives and roots, then the entry's limbs in place of its doubles;
@@ -13,9 +14,11 @@
 //      so a step is straight-line code: with a branch per slot (lane programs) the same sums
 //      left each warp waiting 7 cycles per instruction and the 16-atom medium build took 941 ms
 //      against 811 ms with FP64 lane programs.
-// Measured on that build (CUDA events): (dd|pp) 43.9 -> 24.3 ms, (dd|dp) 56.2 -> 38.2, (dp|dp)
-// 64.8 -> 47.6, (dp|pp) 64.0 -> 54.1, the build 804 -> 708 ms; the FP64 pipe, now with the
-// recurrences and roots, is 91 % busy again.
+// Measured on that build (CUDA events, FP64 class kernel -> this): (dd|pp) 43.9 -> 25.0 ms, (dd|dp) 56.3 ->
+// 39.2, (dp|dp) 64.8 -> 45.9, (pp|pp) 29.2 -> 18.8, (dp|ds) 71.0 -> 60.9, (dp|pp) 64.0 -> 59.2; all
+// nine classes 431 -> 331 ms.  In (dp|dp) the FP64 pipe (recurrences, roots, transfer, digestion)
+// is 49 % busy, the issue slots 52 %: the three warps of a scheduler mostly wait for the fixed
+// latency of dependent integer instructions.
 #include <cuda_runtime.h>
 #include <stdint.h>
 

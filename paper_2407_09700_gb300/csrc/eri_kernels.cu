@@ -22,7 +22,9 @@
 //   3. digestion into J~ and K~ with the six updates of Alg. 2 and the
 //      permutation weights of the unique quartet, by FP64 atomicAdd.
 // Roots and weights are FP64 values of 64-bit fixed-point sums (rys_fixed.h), the recurrences FP64.
-// FP64 J/K launches of classes up to L = 8 run eri_fixed.cu or eri_small.cu instead.
+// FP64 J/K launches of classes up to L = 8 run eri_fixed.cu or eri_small.cu instead, unless a shell pair's
+// exponents spread over more than FX_SPREAD binades; diagonal quartets (Schwarz factors) and
+// eri_shell_quartet run here.
 #include <cuda_runtime.h>
 #include <stdint.h>
 

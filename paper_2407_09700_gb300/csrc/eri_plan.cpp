@@ -1101,7 +1101,8 @@ constexpr long long kListMinTasks = 8192;
 //                 10.6, 12.4; J alone of 27 atoms 27.3 ms; 2, 4, 8, 12 give 28.8, 27.7, 27.5, 27.3
 //   team     80:  5 atoms, spd, UHF 29.0 ms; 8, 24, 80 give 17.5, 15.6, 14.6
 //   gradient 24:  4 atoms with f and g shells 199 ms; 4, 8, 16, 32 give 228, 191, 172, 182;
-//                 5 atoms 5.28 ms; 4, 8, 16, 32 give 6.07, 5.35, 4.79, 4.61
+//                 5 atoms 5.28 ms; 4, 8, 16, 32 give 6.07, 5.35, 4.79, 4.61 (with one copy of the
+//                 gradient to add to; with its 32 copies 24 gives 3.17)
 // Split where the quartet is over the mean load but not over twice it, J alone of 27 atoms is 2 %
 // slower (one-lane 4: 28.3 against 27.7 ms) and nothing else is faster.
 constexpr double FIXED_LANE = 8.0, FIXED_TEAM = 80.0, FIXED_GRAD = 24.0;
@@ -1644,7 +1645,7 @@ eri_status eri_plan_create(const eri_basis* basis, const eri_opts* opts, void* c
           zlo = std::min(zlo, p->prims[sp.prim_off + q].zeta);
           zhi = std::max(zhi, p->prims[sp.prim_off + q].zeta);
         }
-        // unsorted, a batch of a mixed plan holds exponents further apart: 6 binades less allowed
+        // unsorted, a batch of a mixed plan holds exponents further apart: 6 binades less allowed (eri_fixed.cuh)
         const double spread = 0.5 * (p->sh_l[sp.sh0] + p->sh_l[sp.sh1]) * std::log2(zhi / zlo);
         p->type_spread[X] = std::max(p->type_spread[X], spread + (p->opts.precision == ERI_MIXED ? 6.0 : 0.0));
         if (p->sh_l[sp.sh0] > 0) p->type_rt[X] = std::max(p->type_rt[X], fx_zeta(p, sp, zhi) * p->diag2);

@@ -14,7 +14,11 @@
 // 2^-60 per product; "fixed" = units of 2^-60 (or limbs h 2^-30 + l 2^-60), values below 2;
 // lengths of the bra (ket) in units of 2^a (2^b), chosen per primitive pair so that every
 // C = P - A - u eta/(zeta+eta) (P - Q) fits: |C| <= |P - A| + sqrt(c_N / zeta), c_N the largest
-// squared zero of the Hermite polynomial of order 2N (u <= min(1, c_N / T)).
+// squared zero of the Hermite polynomial of order 2N (u <= min(1, c_N / T)).  Weights are held in
+// units of about 1/sqrt(T).  Errors are a few 2^-60 of these units: seven bits below FP64's for
+// values of the units' size, above them for a value whose C's are far below theirs.  SX_TMAX bounds
+// that for tight shells; components that vanish by symmetry, or nearly so, are accurate relative to the
+// unit rather than to themselves.
 #pragma once
 #include <stdint.h>
 

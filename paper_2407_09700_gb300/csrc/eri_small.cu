@@ -1,6 +1,7 @@
 // Compile-time specialised Rys kernels for the low angular-momentum classes whose
 // contracted [e0|f0] block fits a lane's registers (up to 54 values in FP64, 96 in the
-// FP32 path of the mixed mode); each runs with one lane per shell quartet.  Following
+// FP32 path of the mixed mode; in integers sums of more than 30 values live in shared
+// memory); each runs with one lane per shell quartet.  Following
 // Sec. 3's design for small root counts (Alg. 2: unrolled recurrences, intermediates in
 // registers, contraction before digestion), every loop here has compile-time bounds: the
 // 2D tables I_x, I_y, I_z of one root and the contracted accumulators live in registers
@@ -404,7 +405,8 @@ __global__ void __launch_bounds__(TPB, (Small<LA, LB, LC, LD>::NOUT > 32 ? 2 : 3
 // at scale Theta 2^(a |e| + b |f|).  Sums of more than 30 values live in shared memory.
 // The FP64 kernels above kept the FP64 pipe 85 % busy and the integer pipes 10-15 %.  16-atom
 // medium build: (dp|ps) 74.6 -> 50.5 ms, (ds|ps) 47.2 -> 27.8, (ps|ps) 35.3 -> 17.2, (ps|ss) 24.9 ->
-// 9.3, (ss|ss) 5.0 -> 2.7; J and K are as close to quadruple precision as with FP64 (45 functions
+// 9.3, (ss|ss) 6.0 -> 2.5; in (dp|ps) the FP64 pipe is then 36 % busy and two warps a scheduler wait
+// for dependent integer instructions; J and K are as close to quadruple precision as with FP64 (45 functions
 // of 6-31G(d)-like shells: 1.2e-15, 1.6e-15 against 1.3e-15, 1.7e-15 for a small change of the
 // density).
 template <int LA, int LB, int LC, int LD>
