@@ -61,7 +61,7 @@ class Job:
 
 
 def footprint_bytes(mol, kind: str) -> int:
-    """Device memory a job holds while admitted: pair and primitive-pair records,
+    """Device memory a job holds while admitted: pair and primitive-pair records (FP64, FP32, integer),
     density block maxima, D / J / K and (RHF) S, H, X, Fock and DIIS matrices."""
     nsh = int(mol.nshell)
     nbf = int(mol.nbf)
@@ -69,7 +69,7 @@ def footprint_bytes(mol, kind: str) -> int:
     npairs = nsh * (nsh + 1) // 2
     nprim_pairs = int((K.sum() ** 2 + (K ** 2).sum()) // 2)
     mats = 3 + (4 + 2 * 8 + 2 if kind == "scf" else 0)
-    return int(2 * 64 * npairs + (80 + 40) * nprim_pairs + 8 * nsh * nsh + 8 * mats * nbf * nbf + (1 << 20))
+    return int(2 * 64 * npairs + (80 + 32 + 112) * nprim_pairs + 8 * nsh * nsh + 8 * mats * nbf * nbf + (1 << 20))
 
 
 def _percentile(x, q):
