@@ -817,7 +817,7 @@ struct eri_plan {
   int type_maxprim[ERI_NPAIRTYPE] = {0};   // most primitive pairs of a kept pair, per type
   long long type_sumprim[ERI_NPAIRTYPE] = {0};   // primitive pairs of the kept pairs, per type
   double type_spread[ERI_NPAIRTYPE] = {0}; // (l0 + l1) / 2 log2 of the largest ratio of a kept pair's zeta
-  double type_rt[ERI_NPAIRTYPE] = {0};     // l0 + l1 > 0: bound of zeta |P - Q|^2 over the kept pairs (fx_zeta)
+  double type_rt[ERI_NPAIRTYPE] = {0};     // l0 + l1 odd and above 1: bound of zeta |P - Q|^2 over the kept pairs (fx_zeta)
   double diag2 = 0.0;                // squared diagonal of the atoms' bounding box
   int npairs_kept = 0;
   std::vector<double> Q;             // [nshell*nshell]
@@ -1648,7 +1648,8 @@ eri_status eri_plan_create(const eri_basis* basis, const eri_opts* opts, void* c
         // unsorted, a batch of a mixed plan holds exponents further apart: 6 binades less allowed (eri_fixed.cuh)
         const double spread = 0.5 * (p->sh_l[sp.sh0] + p->sh_l[sp.sh1]) * std::log2(zhi / zlo);
         p->type_spread[X] = std::max(p->type_spread[X], spread + (p->opts.precision == ERI_MIXED ? 6.0 : 0.0));
-        if (p->sh_l[sp.sh0] > 0) p->type_rt[X] = std::max(p->type_rt[X], fx_zeta(p, sp, zhi) * p->diag2);
+        const int lsum = p->sh_l[sp.sh0] + p->sh_l[sp.sh1];
+        if (lsum > 1 && lsum % 2) p->type_rt[X] = std::max(p->type_rt[X], fx_zeta(p, sp, zhi) * p->diag2);
       }
     }
     p->type_cnt[X] = (int)kept.size() - p->type_off[X];

@@ -17,18 +17,19 @@
 // squared zero of the Hermite polynomial of order 2N (u <= min(1, c_N / T)).  Weights are held in
 // units of about 1/sqrt(T).  Errors are a few 2^-60 of these units: seven bits below FP64's for
 // values of the units' size, above them for a value whose C's are far below theirs.  SX_TMAX bounds
-// that for tight shells; components that vanish by symmetry, or nearly so, are accurate relative to the
-// unit rather than to themselves.
+// that for tight shells; the smaller components of a quartet, or ones that vanish nearly by symmetry,
+// are accurate relative to its largest rather than to themselves.
 #pragma once
 #include <stdint.h>
 
 #include "eri_internal.h"
 #include "rys_fixed.h"
 
-// Largest zeta |P - Q|^2 of the FP64 launches with p or higher functions.  C of a tight pair on one
-// centre is about 1 / (zeta |P - Q|), sqrt(T) below its unit of length, so that a (ps|ss) carries
-// about 2^-57.6 sqrt(zeta |P - Q|^2): 1.7e-15 at this limit (5.3e-14 measured at 1.3e8, 4.4e-13 at 1.3e10),
-// where FP64 keeps 1e-15.  Wider classes run in FP64.
+// Largest zeta |P - Q|^2 of the FP64 launches with pairs of three or more units of angular momentum, odd in all
+// ((dp| and (fs|).  On one centre, where P - A = 0, each of their values has a factor C, about
+// 1 / (zeta |P - Q|), sqrt(T) below the unit that the half inverse exponent sets, and carries about
+// 2^-57.6 sqrt(zeta |P - Q|^2): 1.7e-15 at this limit, where FP64 keeps 1e-15.  Wider classes run in FP64.  Pairs
+// of even angular momentum have values of the unit's size, and the unit of a (ps| pair goes by C.
 #define SX_TMAX 131072.0
 
 // Fewest binary places of the positions in FP64 and in FP32 launches (64 and 2^28 bohr to either side of
@@ -117,6 +118,18 @@ SX_HD int sx_places(const int64_t c0[3], const int64_t c1[3], int64_t hz) {
   uint64_t m = 0;
   for (int i = 0; i < 3; ++i) m |= (uint64_t)(c0[i] ^ (c0[i] >> 63)) | (uint64_t)(c1[i] ^ (c1[i] >> 63));
   const int p = sx_clz(m) - 4, q = (sx_clz((uint64_t)hz) - 7) >> 1;
+  const int r = p < q ? p : q;
+  return r > 0 ? r : 0;
+}
+
+// Most places p with f 2^(e - 62) < 2^-p; f < 2^62.
+SX_HD int sx_room(int64_t f, int e) { return sx_clz((uint64_t)f) - 2 - e; }
+
+// Most places p with |c| < 2^(59 - p) and f 2^(e - 62) < 2^(-1 - p) (0 if none).
+SX_HD int sx_places1(const int64_t c[3], int64_t f, int e) {
+  uint64_t m = 0;
+  for (int i = 0; i < 3; ++i) m |= (uint64_t)(c[i] ^ (c[i] >> 63));
+  const int p = sx_clz(m) - 5, q = sx_room(f, e) - 1;
   const int r = p < q ? p : q;
   return r > 0 ? r : 0;
 }

@@ -513,7 +513,7 @@ __global__ void __launch_bounds__(TPB, (SmallFx<LA, LB, LC, LD>::blocks)) eri_sm
         const int rze = x.He + s.g2e, ree = y.He + s.g2e;
         const SxL hzl = sx_limbs(x.hz), hel = sx_limbs(y.hz);
         SxL hs{0, 0};
-        if (LE > 0 && LF > 0) {
+        if (LE > 0 && LF > 1) {
           // 1 / (2 (zeta + eta)) 2^-(a + b): from the side that needs no left shift
           const bool br = x.a <= y.a;
           const SxL r = sx_limbs(br ? sx_shift(rem, 2 - ree) : sx_shift(rzm, 2 - rze));
@@ -531,41 +531,64 @@ __global__ void __launch_bounds__(TPB, (SmallFx<LA, LB, LC, LD>::blocks)) eri_sm
           // in units of 2^rTe, about 1/sqrt(T), in the large-T limit: the weight keeps its 60 bits there
           // (as an absolute 2^-60 it lost log2(T) / 2 of them, 2.3e-13 of a repulsion at T = 1e11)
           const int64_t w60 = sx_shift(wm, 2 - (we - s.rTe));
+          // u eta/(zeta+eta), u zeta/(zeta+eta)
+          const int64_t fz = LE > 0 ? sx_mulm(um, rzm) : 0, fn = LF > 0 ? sx_mulm(um, rem) : 0;
+          const int fze = ue + rze, fne = ue + ree;
           int64_t C6[3] = {0, 0, 0}, Cp6[3] = {0, 0, 0}, b10 = 0, b01 = 0, b00 = 0;
-          if (LE > 0) {
-            const int64_t fm = sx_mulm(um, rzm);
-            const int fe = ue + rze;
-            const SxL f = sx_limbs(sx_shift(fm, 2 - (fe + s.k - x.a)));
-#pragma unroll
-            for (int i = 0; i < 3; ++i) C6[i] = x.PA[i] - sx_mul(f, dl[i]);
-            if (LE > 1) b10 = x.hz - sx_mul(hzl, sx_limbs(sx_shift(fm, 2 - fe)));
-          }
-          if (LF > 0) {
-            const int64_t fm = sx_mulm(um, rem);
-            const int fe = ue + ree;
-            const SxL f = sx_limbs(sx_shift(fm, 2 - (fe + s.k - y.a)));
-#pragma unroll
-            for (int i = 0; i < 3; ++i) Cp6[i] = y.PA[i] + sx_mul(f, dl[i]);
-            if (LF > 1) b01 = y.hz - sx_mul(hel, sx_limbs(sx_shift(fm, 2 - fe)));
-          }
-          if (LE > 0 && LF > 0) b00 = sx_mul(hs, sx_limbs(sx_shift(um, 2 - ue)));
           // C is linear in u, so every root's lies between P - A and the largest root's: units in
           // which the larger of them is below 1 and the half inverse exponent below 1/8 (every
           // 2D entry then below 2).  Without this the fourth-degree entries of typical C (a few
           // hundredths of the bound) kept too few bits.
-          if (N > 1 && nn == 0) {
-            if (LE > 0) sa = sx_places(x.PA, C6, x.hz);
-            if (LF > 0) sb = sx_places(y.PA, Cp6, y.hz);
+          if (LE > 1) {
+            const SxL f = sx_limbs(sx_shift(fz, 2 - (fze + s.k - x.a)));
+#pragma unroll
+            for (int i = 0; i < 3; ++i) C6[i] = x.PA[i] - sx_mul(f, dl[i]);
+            b10 = x.hz - sx_mul(hzl, sx_limbs(sx_shift(fz, 2 - fze)));
+            if (N > 1 && nn == 0) sa = sx_places(x.PA, C6, x.hz);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) C6[i] = (int64_t)((uint64_t)C6[i] << sa);
+            b10 = (int64_t)((uint64_t)b10 << (2 * sa));
+          }
+          if (LF > 1) {
+            const SxL f = sx_limbs(sx_shift(fn, 2 - (fne + s.k - y.a)));
+#pragma unroll
+            for (int i = 0; i < 3; ++i) Cp6[i] = y.PA[i] + sx_mul(f, dl[i]);
+            b01 = y.hz - sx_mul(hel, sx_limbs(sx_shift(fn, 2 - fne)));
+            if (N > 1 && nn == 0) sb = sx_places(y.PA, Cp6, y.hz);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) Cp6[i] = (int64_t)((uint64_t)Cp6[i] << sb);
+            b01 = (int64_t)((uint64_t)b01 << (2 * sb));
+            if (LE > 0) b00 = (int64_t)((uint64_t)sx_mul(hs, sx_limbs(sx_shift(um, 2 - ue))) << (sa + sb));
+          }
+          // A side of one unit of angular momentum has no half inverse exponent in its entries: its unit goes
+          // by C alone, before anything is rounded, so that a dipole keeps its bits at any distance
+          // ((ps|ps) of exponents 10 and 1e3 eight bohr apart was off by 2.9e-13 and 3.5e-10)
+          if (LE == 1 && nn == 0) sa = sx_places1(x.PA, fz, fze + s.k - x.a);
+          if (LF == 1) {
+            const int64_t hm = sx_mulm(fz, y.Hm);        // u / (2 (zeta + eta)) = hm 2^(he - 62), units 2^(a + b)
+            const int he = fze + y.He - 1 - x.a - y.a;
+            if (nn == 0) {
+              const int lim = max(0, sx_room(hm, he) - 3);     // places that leave it below 1/8
+              if (LE == 1) sa = sa < lim ? sa : lim;
+              const int p = sx_places1(y.PA, fn, fne + s.k - y.a), q = lim > sa ? lim - sa : 0;
+              sb = p < q ? p : q;
+            }
+            b00 = sx_shift(hm, 2 - (he + sa + sb));
+            const SxL f = sx_limbs(sx_shift(fn, 2 - (fne + s.k - y.a + sb)));
+#pragma unroll
+            for (int i = 0; i < 3; ++i) Cp6[i] = (int64_t)((uint64_t)y.PA[i] << sb) + sx_mul(f, dl[i]);
+          }
+          if (LE == 1) {
+            const SxL f = sx_limbs(sx_shift(fz, 2 - (fze + s.k - x.a + sa)));
+#pragma unroll
+            for (int i = 0; i < 3; ++i) C6[i] = (int64_t)((uint64_t)x.PA[i] << sa) - sx_mul(f, dl[i]);
           }
           SxL C[3], Cp[3];
 #pragma unroll
           for (int i = 0; i < 3; ++i) {
-            C[i] = sx_limbs((int64_t)((uint64_t)C6[i] << sa));
-            Cp[i] = sx_limbs((int64_t)((uint64_t)Cp6[i] << sb));
+            C[i] = sx_limbs(C6[i]);
+            Cp[i] = sx_limbs(Cp6[i]);
           }
-          b10 = (int64_t)((uint64_t)b10 << (2 * sa));
-          b01 = (int64_t)((uint64_t)b01 << (2 * sb));
-          b00 = (int64_t)((uint64_t)b00 << (sa + sb));
           // 2D tables; entry 0 of x and y is 1 and stays out of the products
           SxL g[3][NI];
           g[2][0] = sx_limbs(w60);

@@ -15,6 +15,8 @@ extern "C" {
 
 int64_t host_rsqrt(int64_t f) { return sx_rsqrt(f); }
 
+int host_places1(const int64_t* c, int64_t f, int e) { return sx_places1(c, f, e); }
+
 // H = 1/zeta + 1/eta; out: g, ge, d[3], k, ti, x0, x1, rT, rTe, rT2, g2, g2e
 void host_quartet(double H, const int64_t* P, const int64_t* Q, int pu, int64_t tcut4, int64_t* out) {
   SxQuartet s;

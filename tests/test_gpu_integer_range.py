@@ -23,18 +23,19 @@ def built():
 
 
 def _separated(zeta, R=8.0):
-    """J of an s and a p shell at the origin in the field of an s function at (R, 0, 0): (ss|ss),
-    (px s|ss), (px px|ss) and the values of their multipoles (T = zeta R^2 far above 40, so
-    exponentially small terms are left out)."""
+    """J of an s and a p shell at the origin in the field of an s function, and of a px s and a py s
+    product, at (R, 0, 0): (ss|ss), (px s|ss), (px px|ss), (px s|px s), (py s|py s) and the values of their
+    multipoles (T = zeta R^2 far above 40, so exponentially small terms are left out)."""
     one = np.ones(1)
     m = custom_molecule(np.array([[0.0, 0, 0], [R, 0, 0]]),
-                        [(0, 0, np.array([zeta]), one), (0, 1, np.array([zeta]), one), (1, 0, np.array([zeta]), one)])
-    D = np.zeros((1, m.nbf, m.nbf))
-    D[0, -1, -1] = 1.0
-    J, _ = pkg.Plan(m, tau=0.0).jk(torch.from_numpy(D).cuda())
-    J = J.cpu().numpy()[0]
+                        [(a, l, np.array([zeta]), one) for a in (0, 1) for l in (0, 1)])
+    D = np.zeros((3, m.nbf, m.nbf))
+    D[0, 4, 4] = 1.0
+    D[1, 4, 5] = D[1, 5, 4] = D[2, 4, 6] = D[2, 6, 4] = 0.5
+    J = pkg.Plan(m, tau=0.0).jk(torch.from_numpy(D).cuda())[0].cpu().numpy()
     mu, q = 0.5 / np.sqrt(zeta), 0.25 / zeta      # <s|x|px>; <px|x^2|px> - <px|y^2|px> is 2 q
-    return np.array([J[0, 0], J[0, 1], J[1, 1]]), np.array([1 / R, mu / R ** 2, 1 / R + 2 * q / R ** 3])
+    return (np.array([J[0, 0, 0], J[0, 0, 1], J[0, 1, 1], J[1, 0, 1], J[2, 0, 2]]),
+            np.array([1 / R, mu / R ** 2, 1 / R + 2 * q / R ** 3, -2 * mu ** 2 / R ** 3, mu ** 2 / R ** 3]))
 
 
 # Weights of the large-T limit carry 60 bits relative to 1 / sqrt(T) and everything else about 20
@@ -46,13 +47,14 @@ def test_repulsion_of_tight_shells(zeta):
     assert abs(got[2] / want[2] - 1) <= 4e-15
 
 
-# (ps|ss), a dipole's repulsion, is about 1 / sqrt(zeta R^2) of the unit its C is held in; a few units of
-# 2^-60 leave 2^-57.6 sqrt(zeta R^2), 1.7e-15 at the largest zeta R^2 that the integers take (2^17, between
-# 1e3 and 2e3 here), beside the roundings of the other elements: twice the sum of both.
-@pytest.mark.parametrize("zeta", [1e2, 1e3, 2e3, 1e4, 1e6, 1e8, 1e12])
+# (ps|ss), a dipole's repulsion, is about 1 / sqrt(zeta R^2) of the pair's extent and (ps|ps) 1 / (zeta R^2): their C
+# and the term of both sides are held in units of their own size, so the bound is that of the other
+# elements, doubled for the second C.
+@pytest.mark.parametrize("zeta", [10.0, 1e2, 1e3, 2e3, 1e4, 1e6, 1e8, 1e12])
 def test_dipole_of_tight_shells(zeta):
     got, want = _separated(zeta)
-    assert abs(got[1] / want[1] - 1) <= 8e-15
+    for k in (1, 3, 4):
+        assert abs(got[k] / want[k] - 1) <= 8e-15
 
 
 def _cluster(far, rng):

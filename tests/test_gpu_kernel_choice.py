@@ -79,35 +79,39 @@ def test_spread_of_a_shells_exponents(ratio, mixed, kernel):
         assert np.abs(got - ref).max() <= (2e-14 if kernel == "fixed" else 1e-12) * np.abs(ref).max()
 
 
-# The one-lane integer kernel: up to zeta |P - Q|^2 = 2^17 where p functions are involved, any for s; positions in
+# The one-lane integer kernel: up to zeta |P - Q|^2 = 2^17 for (dp| and (fs| pairs, any for the others; positions in
 # units of 2^-52 bohr, which a box above 128 bohr leaves; exponents within 1e-18 .. 1e18.
-@pytest.mark.parametrize("zeta,R,ss,ps", [(1e3, 8.0, "small_fx", "small_fx"), (2e3, 8.0, "small_fx", "small"),
+@pytest.mark.parametrize("zeta,R,ps,dp", [(1e3, 8.0, "small_fx", "small_fx"), (2e3, 8.0, "small_fx", "small"),
                                           (1.0, 120.0, "small_fx", "small_fx"), (1.0, 130.0, "small", "small"),
-                                          (1e19, 1.0, "small", "small")])
-def test_range_of_the_integer_kernel(zeta, R, ss, ps):
+                                          (1e19, 1.0, "small", None)])
+def test_range_of_the_integer_kernel(zeta, R, ps, dp):
     one = np.ones(1)
-    m = custom_molecule(np.array([[0.0, 0, 0], [R, 0, 0]]), [(a, l, np.array([zeta]), one) for a in (0, 1) for l in (0, 1)])
+    m = custom_molecule(np.array([[0.0, 0, 0], [R, 0, 0]]),
+                        [(a, l, np.array([zeta]), one) for a in (0, 1) for l in ((0, 1, 2) if dp else (0, 1))])
     m.D = random_psd_density(m.nbf, 3, np.random.default_rng(1), 2)
     J, K, kern = _jk(m)
-    assert kern[0, 0, 0, 0] == ss and kern[1, 0, 0, 0] == ps and kern[1, 0, 1, 0] == ps
+    assert all(kern[c] == ps for c in ((0, 0, 0, 0), (1, 0, 0, 0), (1, 0, 1, 0)))
+    if dp:
+        assert kern[2, 0, 0, 0] == ps and kern[2, 1, 0, 0] == dp and kern[2, 1, 1, 0] == dp
     Jr, Kr, _ = oracle.jk(m, tau=0.0)
     for got, ref in ((J, Jr), (K, Kr)):
         assert np.abs(got - ref).max() <= 2e-14 * np.abs(ref).max()
 
 
-# A contracted core s shell (exponents up to 2e4) beside a p shell counts as its diffuse primitives: the integer
-# kernel serves it, and the dipole (px s| in the field of an s function 8 bohr away, where P = A is exact in
-# the oracle too, is as close as that of the single exponents.
+# A contracted core s shell (exponents up to 2e4) beside an f shell counts as its diffuse primitives: the integer
+# kernel serves it, and the dipole (px s| and (fxxx s| in the field of an s function 8 bohr away, where P = A is
+# exact in the oracle too, are as close as those of single exponents.
 def test_contracted_core_stays_in_integers():
     core = np.array([2e4, 3e3, 600.0, 150.0, 40.0, 10.0])
     one = np.ones(1)
     m = custom_molecule(np.array([[0.0, 0, 0], [8.0, 0, 0]]),
                         [(0, 0, core, np.array([0.002, 0.015, 0.07, 0.22, 0.47, 0.36])),
-                         (0, 1, np.array([8.0, 2.0]), np.array([0.4, 0.7])), (1, 0, np.array([0.5]), one)])
+                         (0, 1, np.array([8.0, 2.0]), np.array([0.4, 0.7])), (0, 3, np.array([1.5]), one),
+                         (1, 0, np.array([0.5]), one)])
     m.D = np.zeros((1, m.nbf, m.nbf))
     m.D[0, -1, -1] = 1.0
     J, _, kern = _jk(m)
-    assert kern[1, 0, 0, 0] == "small_fx" and kern[1, 0, 1, 0] == "small_fx"
+    assert kern[3, 0, 0, 0] == "small_fx" and kern[3, 0, 1, 0] == "small_fx"
     Jr, _, _ = oracle.jk(m, tau=0.0)
-    for at in ((0, 0), (0, 1), (1, 1)):
+    for at in ((0, 0), (0, 1), (1, 1), (0, 4)):
         assert abs(J[0][at] / Jr[0][at] - 1) <= 8e-15

@@ -42,6 +42,20 @@ def test_reciprocal_square_root(lib):
         assert abs(lib.host_rsqrt(f) - isqrt((1 << 180) // f)) <= 8
 
 
+def test_places_of_a_sides_unit(lib):
+    # p places leave c (units of 2^-60) and f 2^(e - 62) below a half, one more leaves one of them at a
+    # half or above
+    rng = random.Random(3)
+    for t in range(4000):
+        c = [rng.choice((-1, 1)) * int(2 ** rng.uniform(0, 60)) if rng.random() < 0.7 else 0 for _ in range(3)]
+        f, e = int(2 ** rng.uniform(0, 62)), rng.randrange(-70, 1)
+        p = lib.host_places1((I64 * 3)(*c), I64(f), INT(e))
+        big = max([Fr(abs(x), 1 << 60) for x in c] + [Fr(f) * Fr(2) ** (e - 62)])
+        # a negative c counts as one more than its size does: exact powers of two
+        assert p >= 0 and (p == 0 or big * 2 ** p <= Fr(1, 2))
+        assert big * 2 ** (p + 1) >= Fr(1, 2) or p == 59
+
+
 def test_scalars_of_a_primitive_quartet(lib):
     rng = random.Random(2)
     tcut = 41
