@@ -14,9 +14,9 @@
 //      so a step is straight-line code: with a branch per slot (lane programs) the same sums
 //      left each warp waiting 7 cycles per instruction and the 16-atom medium build took 941 ms
 //      against 811 ms with FP64 lane programs.
-// Measured on that build (CUDA events, FP64 class kernel -> this): (dd|pp) 43.9 -> 25.0 ms, (dd|dp) 56.3 ->
-// 39.2, (dp|dp) 64.8 -> 45.9, (pp|pp) 29.2 -> 18.8, (dp|ds) 71.0 -> 60.9, (dp|pp) 64.0 -> 59.2; all
-// nine classes 431 -> 331 ms.  In (dp|dp) the FP64 pipe (recurrences, roots, transfer, digestion)
+// Measured on that build (CUDA events, FP64 class kernel -> this): (dd|pp) 43.9 -> 24.9 ms, (dd|dp) 56.3 ->
+// 39.0, (dp|dp) 64.8 -> 45.7, (pp|pp) 29.2 -> 18.7, (dp|ds) 71.0 -> 60.7, (dp|pp) 64.0 -> 58.9; all
+// nine classes 430 -> 331 ms.  In (dp|dp) the FP64 pipe (recurrences, roots, transfer, digestion)
 // is 49 % busy, the issue slots 52 %: the three warps of a scheduler mostly wait for the fixed
 // latency of dependent integer instructions.
 #include <cuda_runtime.h>

@@ -404,8 +404,8 @@ __global__ void __launch_bounds__(TPB, (Small<LA, LB, LC, LD>::NOUT > 32 ? 2 : 3
 // each primitive quartet's sums over the roots return to FP64 (a conversion and an FMA per value)
 // at scale Theta 2^(a |e| + b |f|).  Sums of more than 30 values live in shared memory.
 // The FP64 kernels above kept the FP64 pipe 85 % busy and the integer pipes 10-15 %.  16-atom
-// medium build: (dp|ps) 74.6 -> 50.5 ms, (ds|ps) 47.2 -> 27.8, (ps|ps) 35.3 -> 17.2, (ps|ss) 24.9 ->
-// 9.3, (ss|ss) 6.0 -> 2.5; in (dp|ps) the FP64 pipe is then 36 % busy and two warps a scheduler wait
+// medium build: (dp|ps) 74.5 -> 49.7 ms, (ds|ps) 47.2 -> 26.4, (ps|ps) 35.3 -> 15.6, (ps|ss) 24.9 ->
+// 9.5, (ss|ss) 6.0 -> 2.5; in (dp|ps) the FP64 pipe is then 36 % busy and two warps a scheduler wait
 // for dependent integer instructions; J and K are as close to quadruple precision as with FP64 (45 functions
 // of 6-31G(d)-like shells: 1.2e-15, 1.6e-15 against 1.3e-15, 1.7e-15 for a small change of the
 // density).
